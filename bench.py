@@ -178,7 +178,7 @@ class ClockSampler:
 
 
 # profiler kernel ids -> CUDA kernels whose ncu DRAM traffic profiles/dram_traffic.md records
-TRAFFIC_KERNEL = {"stars": "k_star_stream", "spmv": "k_spmv_dir", "update": "k_update",
+TRAFFIC_KERNEL = {"stars": "k_star_solve", "spmv": "k_spmv_dir", "update": "k_update",
                   "combine": "k_combine", "coarse": "k_coarse_symv"}
 
 
@@ -243,8 +243,8 @@ def kernel_bytes(op, pc, prec_bytes):
     solve that is the gather of r and the write of the local results (an index
     list, r and the result: 4 + 8 + 8 bytes per star entry) and the factor
     coefficients of both triangular solves (2 v per entry of L, diagonal
-    included); its window descriptors, column indices, padding slots, star
-    headers and inverse permutations are format overhead.  For the coarse
+    included); its step and group headers, column indices, padding, star headers
+    and inverse permutations are format overhead.  For the coarse
     solve it is the upper triangle of the symmetric A_0^{-1} (the dense-inverse
     method), the tile padding being overhead; int64 row pointers count as int32.
     """
@@ -277,7 +277,7 @@ def kernel_bytes(op, pc, prec_bytes):
         "spmv": 4 * (n + 1),
         "update": 0,
         "coarse": tiles - vb * m0 * (m0 + 1) // 2,
-        # the solve streams as stored (window records, headers, inverse permutations), r and
+        # the solve data as stored (records, headers, inverse permutations), r and
         # the results, less the algorithmic bytes
         "stars": int(i.star_stream_bytes + 8 * ss + vb * ss - alg["stars"]),
         "combine": 0,

@@ -45,9 +45,9 @@ extern "C" {
 #define SPNET_ERR_NOT_SPD (-2)         /* a pivot <= 0 in a local or coarse factorisation */
 #define SPNET_ERR_NO_MEMORY (-3)       /* device allocation failed */
 #define SPNET_ERR_NO_CONVERGENCE (-4)  /* maxit reached; the iterate is still returned */
-#define SPNET_ERR_TIMEOUT (-5)         /* a bounded device wait expired (reserved: no call of
-                                          this build waits on the device with a limit, so
-                                          none returns it) */
+#define SPNET_ERR_TIMEOUT (-5)         /* a bounded device wait expired: a star solve gave up
+                                          on a copy of its factor data (2 s); the result of
+                                          the call is not valid */
 #define SPNET_ERR_CUDA (-6)            /* a CUDA runtime error */
 #define SPNET_ERR_UNSUPPORTED (-7)     /* a size beyond the limits of this build */
 #define SPNET_ERR_BAD_H (-8)           /* l_i / H is not an integer >= 1 */
@@ -101,16 +101,15 @@ typedef struct {
                         memory), each right-hand side with its own scalars and stop test;
                         the matrix, the star factors and the coarse tiles are read once
                         per block */
-  int star_map;      /* warps per block of the one-vector star solve: 0 picks it per size
-                        class (stars, largest star, entries per star) by timing the candidates
-                        once per process (default); 1..8 fixes it.  Every warp solves whole
-                        stars, so the choice changes no result */
+  int star_map;      /* warps that solve a star together in the one-vector star solve: 0 picks
+                        it per size class (stars, largest star, bytes per star) by timing the
+                        candidates once per process (default); 1..8 fixes it.  A row is one
+                        lane's sum whatever the warps, so the choice changes no result */
   int patch;         /* SPNET_PATCH_* (default SPNET_PATCH_ELEMENT) */
-  int no_panels;     /* 1: solve the dense block that ends a large star's elimination level by
-                        level also in blocks of right-hand sides; 0 (default): in mixed
-                        precision with batch_rhs >= 2, blocks of 32 nodes or more are solved
-                        by 16-row panels with tensor-core products (TF32 inputs split in high
-                        and low parts, FP32 accumulation) */
+  int no_panels;     /* 1: the dense block that ends a star's elimination is solved a node a
+                        level; 0 (default): it is kept as its FP64 inverse, rounded to the
+                        solve's precision, and applied as one product (a block too
+                        ill-conditioned for that is solved a node a level all the same) */
   int coarse_space;  /* SPNET_COARSE_* (default SPNET_COARSE_Q1) */
   int reserved[7];
 } spnet_options;
@@ -145,15 +144,16 @@ typedef struct {
   int precision, star_set, flexible;
   double setup_ms;      /* device time of setup_preconditioner */
   int64_t device_bytes; /* device memory held by the preconditioner */
-  int64_t star_stream_bytes; /* bytes one star solve reads from its solve streams
-                                (headers, inverse permutations, entries) */
-  int64_t star_warps_per_block; /* the star solve's mapping in use (see spnet_options.star_map) */
+  int64_t star_stream_bytes; /* bytes one star solve reads of its factors
+                                (headers, places, records) */
+  int64_t star_warps_per_block; /* warps per star in use (see spnet_options.star_map) */
   int64_t coarse_dropped;       /* coarse functions left out of A_0^{-1} as linear combinations
                                    of earlier ones (see setup_preconditioner) */
-  int64_t panel_stars;          /* stars whose dense block the k-right-hand-side solve runs by
-                                   panels on tensor cores (see spnet_options.no_panels) */
+  int64_t panel_stars;          /* stars whose dense block of 32 or more nodes blocks of
+                                   right-hand sides apply as its inverse (mixed precision,
+                                   batch_rhs >= 2; see spnet_options.no_panels) */
   int64_t tuned;                /* the tuner's other choices: SpMV lanes per row
-                                   + 256 * right-hand sides per warp of the batched star solve
+                                   + 256 * right-hand sides per team of the batched star solve
                                    (0: chosen by the block width) */
 } spnet_pc_info;
 
@@ -339,10 +339,10 @@ int spnet_server_budget(spnet_server_t server, int64_t* bytes);
 int spnet_server_destroy(spnet_server_t server);
 
 /* The tuner.  setup_preconditioner times, once per device and size class, the warps per
- * block of the one-vector star solve (unless spnet_options.star_map fixes it), the lanes
+ * star of the one-vector star solve (unless spnet_options.star_map fixes it), the lanes
  * per row of the SpMV (operators of 65536 free dofs or more) and the right-hand sides per
- * warp of the batched star solve (batch_rhs >= 4), on the preconditioner's own data, and
- * keeps the choices in a process-wide cache.  The last two change the order of sums, so
+ * team of the batched star solve (batch_rhs >= 4), on the preconditioner's own data, and
+ * keeps the choices in a process-wide cache.  The lanes change the order of sums, so
  * every set-up of a class uses the one measured value (a set-up meeting a class being
  * measured waits for it).  The cache can be saved and loaded, so that another process takes
  * the same choices without measuring: a text file of lines

@@ -31,6 +31,7 @@ struct BScal {
   int done[KMAX], iters[KMAX];
   double rtol;
   int k, maxit, iter, all_done;
+  int err;  // a bounded device wait of the star solves ran out
   unsigned cnt[4];
 };
 
@@ -442,7 +443,7 @@ static void launch_bspmm(spnet_pc_s* pc, Batch& b, cudaStream_t s) {
 static int precond_batch(spnet_pc_s* pc, Batch& b, cudaStream_t s) {
   launch_bupdate(pc, b, 1, s);
   SPNET_TRY(launch_coarse_batch(pc, b.EP, b.k, b.ZC, b.cpart, nullptr, s));
-  SPNET_TRY(launch_star_batch(pc, b.R, b.k, b.W, nullptr, s));
+  SPNET_TRY(launch_star_batch(pc, b.R, b.k, b.W, &b.bs->err, nullptr, s));
   launch_bcombine(pc, b, 2, s);
   return SPNET_OK;
 }
@@ -454,10 +455,10 @@ static int batch_iteration(spnet_pc_s* pc, Batch& b, cudaStream_t s, cudaStream_
   if (side) {
     SPNET_CUDA_TRY(cudaEventRecord(b.ev_fork, s));
     SPNET_CUDA_TRY(cudaStreamWaitEvent(side, b.ev_fork, 0));
-    SPNET_TRY(launch_star_batch(pc, b.R, b.k, b.W, done, side));
+    SPNET_TRY(launch_star_batch(pc, b.R, b.k, b.W, &b.bs->err, done, side));
     SPNET_CUDA_TRY(cudaEventRecord(b.ev_join, side));
   } else {
-    SPNET_TRY(launch_star_batch(pc, b.R, b.k, b.W, done, s));
+    SPNET_TRY(launch_star_batch(pc, b.R, b.k, b.W, &b.bs->err, done, s));
   }
   SPNET_TRY(launch_coarse_batch(pc, b.EP, b.k, b.ZC, b.cpart, done, s));
   if (side) SPNET_CUDA_TRY(cudaStreamWaitEvent(s, b.ev_join, 0));
@@ -486,12 +487,15 @@ int pc_apply_batch_free(spnet_pc_s* pc, int k, const double* r, double* z, int w
   const int wc = which != 2, ws = which != 1;
   launch_bupdate(pc, b, 1, s);
   if (wc) SPNET_TRY(launch_coarse_batch(pc, b.EP, b.k, b.ZC, b.cpart, nullptr, s));
-  if (ws) SPNET_TRY(launch_star_batch(pc, b.R, b.k, b.W, nullptr, s));
+  if (ws) SPNET_TRY(launch_star_batch(pc, b.R, b.k, b.W, &b.bs->err, nullptr, s));
   launch_bcombine(pc, b, 0, s, wc, ws);
   note_launch();
   k_cols_from_pc<<<pc->G, 256, 0, s>>>(N, k, pc->perm, b.Z, z);
+  int err = 0;
+  SPNET_CUDA_TRY(cudaMemcpyAsync(&err, &b.bs->err, sizeof(int), cudaMemcpyDeviceToHost, s));
   SPNET_CUDA_TRY(cudaStreamSynchronize(s));
   SPNET_CUDA_TRY(cudaGetLastError());
+  if (err) return fail(SPNET_ERR_TIMEOUT, "spnet_pc_apply_batch: a device wait of the star solves ran out");
   return SPNET_OK;
 }
 
@@ -610,6 +614,7 @@ int pcg_batch_run(spnet_op_s* op, spnet_pc_s* pc, int k, const double* df, const
       }
       SPNET_CUDA_TRY(cudaMemcpyAsync(&h, b.bs, sizeof(BScal), cudaMemcpyDeviceToHost, s));
       SPNET_CUDA_TRY(cudaStreamSynchronize(s));
+      if (h.err) return fail(SPNET_ERR_TIMEOUT, "pcg_solve: a device wait of the star solves ran out");
       if (h.all_done) break;
     }
   }

@@ -86,6 +86,7 @@ struct Csr {
 struct Scal {
   double rz, pq, rr, bb, alpha, beta, rr_true, rtol;
   int maxit, iter, done, restarts;
+  int err;          // a bounded device wait of the star solves ran out
   unsigned cnt[4];  // arrival counters of the last-block reductions
 };
 
@@ -185,27 +186,27 @@ struct spnet_pc_s {
   int32_t* star_lev = nullptr;     // [S]
   int32_t* star_nnz = nullptr;     // [S]
   int32_t* star_core = nullptr;    // [S] nodes of the dense block that ends each star's elimination
-  // k-right-hand-side solves (FP32) of stars whose dense block is solved by panels on tensor cores
-  int panels = 1;                  // build them (spnet_options.panels)
-  int panel_stars = 0;             // stars solved that way
-  void* bhdr = nullptr;            // [S] headers of the k-right-hand-side solve (null: none)
-  char* brec = nullptr;            // their window records
-  float* coreL = nullptr;          // the dense blocks' tiles in MMA fragment order
-  int64_t panel_bytes = 0;         // bytes of brec and coreL
-  // solve windows: per-star header (80 B), inverse permutation, window records
+  int panels = 1;                  // invert the dense blocks (spnet_options.no_panels = 0)
+  int core_inv = 0;                // largest dense block that is inverted
+  int panel_stars = 0;             // stars whose block of 32 or more nodes a batched solve applies so
+  std::vector<int32_t> star_inv;   // [S] host: nodes of each star's inverted dense block (0: none)
+  // solve records (starsolve.cu)
   void* shdr = nullptr;            // [S] headers
-  uint16_t* iperm_star = nullptr;  // [sum_s] local index -> elimination position, at star_ptr
-  char* srec = nullptr;            // [n_entries] window records (208 B FP32, 336 B FP64)
-  int64_t n_entries = 0;           // window records of all stars
+  uint16_t* iperm_star = nullptr;  // [sum_s] local index -> place in the solve's vector, at star_ptr
+  char* srec = nullptr;            // the records of all stars
+  uint32_t* rec_off = nullptr;     // per star its records' offsets (16 B units), one past the last
+  int64_t* core_off = nullptr;     // [S] byte offset of each star's inverse in srec (set-up only)
+  int32_t* core_kc = nullptr;      // [S] columns per record of it (set-up only)
+  void* rec_counts = nullptr;      // [S] record counts (set-up only, as the next three)
+  int32_t* rec_place = nullptr;    // [S] place of each star in the order of the blocks
+  int64_t *rec_first = nullptr, *rec_base = nullptr;  // [S+1] first entry in rec_off, first byte in srec
+  uint16_t* ford = nullptr;        // [sum_s] rows of each level by forward entries (set-up only)
+  uint16_t* bord = nullptr;        // [sum_s] the same by backward entries
+  int64_t srec_bytes = 0;
+  int rec_size = 0;                // largest record, bytes
+  int ylen = 0;                    // longest solve vector (entries)
   int64_t stream_bytes = 0;        // bytes one solve reads from headers, permutations and records
-  int solve_wpb = 0;               // warps (stars) per block of the solve
-  int solve_blocks = 0;            // blocks of the solve (a multiple of the SM count)
-  size_t solve_smem = 0;           // its dynamic shared memory per block
-  int32_t* sorder = nullptr;       // [solve_blocks*solve_wpb] star of each warp slot, -1: idle
-  int32_t* star_desc = nullptr;    // [S] stars by solve cost, largest first
-  std::vector<double> star_cost;   // [S] host: estimated solve cost of each star
-  std::vector<int32_t> star_ord;   // [S] host: stars by cost, largest first
-  int solve_wpb_max = 0;           // most warps per block the shared-memory budget holds
+  int solve_wpb = 0;               // warps that solve a star together (one block per star)
   // work vectors (pc order)
   double *x = nullptr, *r = nullptr, *p = nullptr, *q = nullptr, *z = nullptr, *b = nullptr;
   double* r2 = nullptr;            // second residual buffer (the iterations alternate)
@@ -288,6 +289,8 @@ inline Mesh mesh_of_pc(const spnet_pc_s* pc) {
 
 constexpr int RED_BLOCK = 256;
 constexpr int A0_KEEP = 2048;
+constexpr int64_t STAR_HUGE = 150 * 1024;  // bytes of a star's solve vector past which records and
+                                           // inverted blocks are kept small (shared memory)
 
 // util.cu
 enum KernelId {
@@ -330,10 +333,11 @@ int pc_galerkin(spnet_pc_s* pc, double* A0_dense);
 // starfact.cu
 int pc_factor_stars(spnet_pc_s* pc);
 // star solves for k <= 32 right-hand sides at once (R, W: [dofs][k]); W in the solve precision
-int launch_star_batch(spnet_pc_s* pc, const double* R, int k, void* W, const int* done, cudaStream_t s);
-// the largest block width (a power of two <= 32) whose star solve fits a block's shared memory
+// (err: set where a wait ran out)
+int launch_star_batch(spnet_pc_s* pc, const double* R, int k, void* W, int* err, const int* done, cudaStream_t s);
+// the largest block width whose star solve fits a block's shared memory
 int star_batch_max_k(const spnet_pc_s* pc);
-// the star solve's mapping (warps per block): fixed by the options, or tuned per size class
+// the star solve's mapping (warps per star): fixed by the options, or tuned per size class
 int star_map_tune(spnet_pc_s* pc);
 // coarse solve for k <= 32 right-hand sides at once: ZC [m0][k] from the corner sums EP [entries][k]
 size_t coarse_batch_part_bytes(const spnet_pc_s* pc, int k);
@@ -423,7 +427,7 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;\
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
 
 // launch with programmatic stream serialization: the kernel may start while
-// the previous kernel of the stream finishes (it must call pdl_wait first)
+// the previous kernel of the stream finishes (it must call pdl_wait first).
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
                               Args&&... args) {
