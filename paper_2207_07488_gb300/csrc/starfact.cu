@@ -96,7 +96,7 @@ struct StarArgs {
   char* scratch;
   int64_t stride;  // global scratch bytes per warp
   int64_t hot;     // hot bytes per warp
-  int hot_in_smem; // 1: hot arrays in dynamic shared memory
+  int hot_in_smem; // 1: degrees, states and marks in dynamic shared memory (k_star_symbolic_block)
   int nmax;
   int core_max;    // largest dense block the scratch holds
   char* pool;
@@ -205,7 +205,7 @@ __global__ void __launch_bounds__(128) k_star_symbolic(StarArgs A) {
   const int lane = threadIdx.x & 31;
   const int64_t wg = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   char* cold = A.scratch + wg * A.stride;
-  char* hot = A.hot_in_smem ? sm_hot + (threadIdx.x >> 5) * A.hot : cold + cold_bytes(A.nmax, A.core_max, A.cap);
+  char* hot = sm_hot + (threadIdx.x >> 5) * A.hot;
   const Scratch W = carve(cold, hot, A.nmax, A.core_max, A.cap);
   const int CAP = A.cap, SWITCH_DEG = switch_degree(A.cap);
   const unsigned FULL = 0xffffffffu;
@@ -522,6 +522,371 @@ __global__ void __launch_bounds__(128) k_star_symbolic(StarArgs A) {
   }
 }
 
+// ---------------------------------------------------------------------------
+// The same for stars whose adjacency lists do not fit shared memory: a block of four warps per
+// star.  Lists lie in global scratch; degrees, states and marks in shared memory where they fit.
+// The fill of a round is added list by list instead of pair by pair: a warp takes an alive
+// neighbour of the eliminated nodes, drops those from its list and appends the entries of their
+// columns that it does not hold yet, told by a bitmap of the star's nodes in shared memory.  A
+// list has one writer and nothing is looked up in another node's list.  (A warp per star, a pair
+// at a time with a search of one member's list, is bound by the latency of those searches: 12.7
+// ms on a 119,000-node 2D network, 16.4 ms on the structural workload.)
+// ---------------------------------------------------------------------------
+constexpr int BT = 128;  // threads of a block
+
+__host__ __device__ inline int64_t bitmap_bytes(int nmax) { return align_up((int64_t)(nmax + 31) / 32 * 4, 16); }
+__host__ __device__ inline int64_t marks_bytes(int nmax) { return align_up(9ll * nmax, 16); }  // deg, state, sel
+
+struct BlockScan {  // per-warp totals
+  int a[BT / 32], b[BT / 32];
+};
+
+__global__ void __launch_bounds__(BT) k_star_symbolic_block(StarArgs A) {
+  extern __shared__ __align__(16) char sm_hot[];
+  __shared__ BlockScan bsc;
+  __shared__ int sh_i[2];
+  __shared__ unsigned long long sh_off;
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  char* cold = A.scratch + (int64_t)blockIdx.x * A.stride;
+  Scratch W = carve(cold, cold + cold_bytes(A.nmax, A.core_max, A.cap), A.nmax, A.core_max, A.cap);
+  uint32_t* bm = (uint32_t*)(sm_hot + wid * bitmap_bytes(A.nmax));
+  if (A.hot_in_smem) {
+    char* p = sm_hot + (BT / 32) * bitmap_bytes(A.nmax);
+    W.deg = (int32_t*)p;
+    W.state = W.deg + A.nmax;
+    W.sel = (uint8_t*)(W.state + A.nmax);
+  }
+  const int CAP = A.cap, SWITCH_DEG = switch_degree(A.cap);
+  constexpr unsigned FULL = 0xffffffffu;
+  for (int i = lane; i < (A.nmax + 31) / 32; i += 32) bm[i] = 0;
+  // exclusive prefix over the block of (on ? 1 : 0, v), and the totals; every thread calls
+  auto scan = [&](bool on, int v, int& before_n, int& before_v, int& tot_n, int& tot_v) {
+    const unsigned b = __ballot_sync(FULL, on);
+    const int incl = warp_incl_scan(v, lane);
+    if (lane == 31) {
+      bsc.a[wid] = __popc(b);
+      bsc.b[wid] = incl;
+    }
+    __syncthreads();
+    before_n = __popc(b & ((1u << lane) - 1u));
+    before_v = incl - v;
+    tot_n = tot_v = 0;
+#pragma unroll
+    for (int w = 0; w < BT / 32; ++w) {
+      if (w < wid) {
+        before_n += bsc.a[w];
+        before_v += bsc.b[w];
+      }
+      tot_n += bsc.a[w];
+      tot_v += bsc.b[w];
+    }
+    __syncthreads();
+  };
+  for (;;) {
+    if (tid == 0) sh_i[0] = atomicAdd(A.next, 1);
+    __syncthreads();
+    const int s = sh_i[0];
+    if (s >= A.S) break;
+    const int k = A.star_mesh[s];
+    const int n = A.star_n[s];
+    const StarElems se = star_elems(A.m, k, A.elem_ptr);
+    int km[3];
+    mesh_multi(A.m, k, km);
+    const bool sup = A.patch == SPNET_PATCH_SUPPORT;
+    // adjacency of the star graph (off-support dofs are isolated nodes, as above)
+    for (int t = tid; t < n; t += BT) {
+      const int i = pc_of_local(se, A.elem_ptr, t);
+      int cnt = 0;
+      bool o = false;
+      const bool tex = sup && off_support(se, A.elem_ptr, A.q1w, A.N, t);
+      for (int64_t q = tex ? A.kptr[i + 1] : A.kptr[i]; q < A.kptr[i + 1]; ++q) {
+        const int j = A.kcol[q];
+        if (j == i) continue;
+        const int lt = local_of_pc(A.m, se, A.elem_ptr, A.elem_of, km[0], km[1], km[2], j);
+        if (lt < 0) continue;
+        if (sup && off_support(se, A.elem_ptr, A.q1w, A.N, lt)) continue;
+        if (cnt < CAP) W.nbr[(int64_t)t * CAP + cnt++] = (uint16_t)lt;
+        else o = true;
+      }
+      W.deg[t] = cnt;
+      W.state[t] = o ? ST_FROZEN : -1;
+    }
+    __syncthreads();
+    int npos = 0, nlev = 0, ncol = 0;
+    bool dense = false;
+    const int core_inv = A.noinv[s] ? 0 : A.core_inv;
+    const int tail = core_inv > 0 ? tail_nodes(n) : 0;
+    while (npos < n) {
+      if (n - npos <= tail) {
+        dense = true;
+        break;
+      }
+      int md = 1 << 30;  // over the nodes that may still be eliminated
+      for (int t = tid; t < n; t += BT)
+        if (W.state[t] == -1) md = min(md, W.deg[t]);
+      md = warp_min(md);
+      if (lane == 0) bsc.a[wid] = md;
+      __syncthreads();
+      md = min(min(bsc.a[0], bsc.a[1]), min(bsc.a[2], bsc.a[3]));
+      if (md > SWITCH_DEG) {
+        dense = true;
+        __syncthreads();
+        break;
+      }
+      const int thr = round_degree(md, SWITCH_DEG);
+      // independent set: candidates of degree <= thr that beat every candidate neighbour
+      for (int t = tid; t < n; t += BT) {
+        bool sl = false;
+        if (W.state[t] == -1 && W.deg[t] <= thr) {
+          sl = true;
+          const int dt = W.deg[t];
+          const uint32_t ht = node_rank(t);
+          const uint16_t* lst = W.nbr + (int64_t)t * CAP;
+          for (int q = 0; q < dt; ++q) {
+            const int u = lst[q];
+            const int du = W.deg[u];
+            if (W.state[u] == -1 && du <= thr && (du < dt || (du == dt && node_rank(u) < ht))) {
+              sl = false;
+              break;
+            }
+          }
+        }
+        W.sel[t] = sl ? 1 : 0;
+      }
+      __syncthreads();
+      // positions in ascending node order, columns = current neighbour lists
+      const int lev_start = npos;
+      if (tid == 0) W.lvl[nlev] = npos;
+      for (int base = 0; base < n; base += BT) {
+        const int t = base + tid;
+        const bool sl = t < n && W.sel[t] == 1;
+        const int dcount = sl ? W.deg[t] : 0;
+        int bn, bv, tn, tv;
+        scan(sl, dcount, bn, bv, tn, tv);
+        if (sl) {
+          const int pos = npos + bn, cs = ncol + bv;
+          W.posnode[pos] = t;
+          W.colstart[pos] = cs;
+          const uint16_t* lst = W.nbr + (int64_t)t * CAP;
+          for (int q = 0; q < dcount; ++q) W.colent[cs + q] = lst[q];
+          W.state[t] = pos;
+        }
+        npos += tn;
+        ncol += tv;
+      }
+      if (tid == 0) W.colstart[npos] = ncol;
+      __syncthreads();
+      // the alive neighbours of the eliminated nodes, each marked once
+      for (int q = W.colstart[lev_start] + tid; q < ncol; q += BT) W.sel[W.colent[q]] = 2;
+      __syncthreads();
+      for (int base = wid * 32; base < n; base += BT) {
+        const int t0 = base + lane;
+        unsigned todo = __ballot_sync(FULL, t0 < n && W.sel[t0] == 2 && W.state[t0] == -1);
+        while (todo) {
+          const int a = base + __ffs(todo) - 1;
+          todo &= todo - 1;
+          uint16_t* lst = W.nbr + (int64_t)a * CAP;
+          const int d = W.deg[a];
+          constexpr int MB = CAP_MAX / 32;
+          int ent[MB], est[MB];
+#pragma unroll
+          for (int b = 0; b < MB; ++b) {
+            const int q = b * 32 + lane;
+            ent[b] = q < d ? lst[q] : -1;
+            est[b] = ent[b] >= 0 ? W.state[ent[b]] : -1;
+          }
+          __syncwarp();
+          if (lane == 0) atomicOr(&bm[a >> 5], 1u << (a & 31));
+          int cnt = 0;
+#pragma unroll
+          for (int b = 0; b < MB; ++b) {  // kept entries move up, in order
+            const bool keep = ent[b] >= 0 && est[b] < 0;
+            const unsigned bal = __ballot_sync(FULL, keep);
+            if (keep) {
+              lst[cnt + __popc(bal & ((1u << lane) - 1u))] = (uint16_t)ent[b];
+              atomicOr(&bm[ent[b] >> 5], 1u << (ent[b] & 31));
+            }
+            cnt += __popc(bal);
+          }
+          __syncwarp();
+#pragma unroll
+          for (int b = 0; b < MB; ++b) {  // the columns of the eliminated ones
+            unsigned gone = __ballot_sync(FULL, ent[b] >= 0 && est[b] >= 0);
+            while (gone) {
+              const int src = __ffs(gone) - 1;
+              gone &= gone - 1;
+              const int pos = __shfl_sync(FULL, est[b], src);
+              const int ce = W.colstart[pos + 1];
+              for (int q0 = W.colstart[pos]; q0 < ce; q0 += 32) {
+                const int u = q0 + lane < ce ? W.colent[q0 + lane] : -1;
+                const bool add = u >= 0 && !((bm[u >> 5] >> (u & 31)) & 1u);
+                const unsigned bal = __ballot_sync(FULL, add);
+                if (add) {
+                  const int at = cnt + __popc(bal & ((1u << lane) - 1u));
+                  if (at < CAP) {
+                    lst[at] = (uint16_t)u;
+                    atomicOr(&bm[u >> 5], 1u << (u & 31));
+                  }
+                }
+                cnt += __popc(bal);
+                __syncwarp();
+              }
+            }
+          }
+          // a list past its slots: the node waits for the dense block (entries that did not fit
+          // set no bit)
+          if (lane == 0) {
+            W.deg[a] = cnt < CAP ? cnt : CAP;
+            if (cnt > CAP) W.state[a] = ST_FROZEN;
+            bm[a >> 5] = 0;
+          }
+          const int dn = cnt < CAP ? cnt : CAP;
+          for (int q = lane; q < dn; q += 32) bm[lst[q] >> 5] = 0;
+          __syncwarp();
+        }
+      }
+      __syncthreads();
+      nlev++;
+    }
+    auto place_rest = [&](bool off_only) {
+      for (int base = 0; base < n; base += BT) {
+        const int t = base + tid;
+        const bool al = t < n && W.state[t] < 0 && (!off_only || off_support(se, A.elem_ptr, A.q1w, A.N, t));
+        int bn, bv, tn, tv;
+        scan(al, 0, bn, bv, tn, tv);
+        if (al) {
+          W.posnode[npos + bn] = t;
+          W.colstart[npos + bn] = ncol;
+          W.state[t] = npos + bn;
+        }
+        npos += tn;
+      }
+    };
+    if (dense && npos < n && sup) {  // off-support dofs left: a level of their own
+      const int p0 = npos;
+      place_rest(true);
+      if (npos > p0) {
+        if (tid == 0) {
+          W.lvl[nlev] = p0;
+          W.colstart[npos] = ncol;
+        }
+        nlev++;
+      }
+      __syncthreads();
+    }
+    int core_c = 0;    // nodes of the dense block
+    bool inv = false;  // it is inverted: no columns, no levels
+    if (dense && npos < n) {
+      const int core0 = npos, c = n - core0;
+      core_c = c;
+      inv = c <= core_inv;
+      if (!inv && (c > A.core_max || ncol + core_entries(c) > (int64_t)A.nmax * CAP + core_entries(A.core_max))) {
+        if (tid == 0) atomicOr(A.flags, FLAG_STAR_BIG);
+        __syncthreads();
+        continue;
+      }
+      place_rest(false);
+      __syncthreads();
+      if (inv) {
+        if (tid == 0) W.colstart[n] = ncol;
+      } else {
+        for (int q = wid; q < c; q += BT / 32) {
+          const int cs = ncol + q * (c - 1) - q * (q - 1) / 2;
+          if (lane == 0) {
+            W.lvl[nlev + q] = core0 + q;
+            W.colstart[core0 + q] = cs;
+          }
+          for (int r = q + 1 + lane; r < c; r += 32) W.colent[cs + (r - q - 1)] = (uint16_t)W.posnode[core0 + r];
+        }
+        nlev += c;
+        ncol += c * (c - 1) / 2;
+        if (tid == 0) W.colstart[n] = ncol;
+      }
+    }
+    if (tid == 0) W.lvl[nlev] = inv ? n - core_c : n;
+    // column entries to positions; row counts and starts
+    for (int t = tid; t <= n; t += BT) W.rcnt[t] = 0;
+    __syncthreads();
+    for (int q = tid; q < ncol; q += BT) {
+      const int pos = W.state[W.colent[q]];
+      W.colent[q] = (uint16_t)pos;
+      atomicAdd(&W.rcnt[pos], 1);
+    }
+    __syncthreads();
+    int carry = 0;
+    for (int base = 0; base < n; base += BT) {
+      const int t = base + tid;
+      int bn, bv, tn, tv;
+      scan(false, t < n ? W.rcnt[t] : 0, bn, bv, tn, tv);
+      if (t < n) W.rstart[t] = carry + bv;
+      carry += tv;
+    }
+    if (tid == 0) W.rstart[n] = carry;
+    for (int t = tid; t < n; t += BT) W.rcnt[t] = 0;
+    // place the blob
+    const BlobLayout L = blob_layout(n, nlev, ncol);
+    if (tid == 0) sh_off = atomicAdd(A.pool_top, (unsigned long long)L.total);
+    __syncthreads();
+    const unsigned long long off = sh_off;
+    if ((int64_t)off + L.total > A.pool_cap) {
+      if (tid == 0) atomicOr(A.flags, FLAG_POOL);
+      __syncthreads();
+      continue;
+    }
+    char* blob = A.pool + off;
+    if (tid == 0) {
+      int32_t* hdr = (int32_t*)blob;
+      hdr[0] = n;
+      hdr[1] = nlev;
+      hdr[2] = ncol;
+      hdr[3] = inv ? core_c : 0;
+      A.star_off[s] = (int64_t)off;
+      A.star_lev[s] = nlev + (inv ? 1 : 0);
+      A.star_nnz[s] = ncol;
+      A.star_core[s] = core_c;
+    }
+    int32_t* gidx = (int32_t*)(blob + L.gidx);
+    uint16_t* perm = (uint16_t*)(blob + L.perm);
+    uint16_t* lvl = (uint16_t*)(blob + L.lvl);
+    uint32_t* colptr = (uint32_t*)(blob + L.colptr);
+    uint16_t* colidx = (uint16_t*)(blob + L.colidx);
+    uint32_t* rowptr = (uint32_t*)(blob + L.rowptr);
+    uint16_t* rowidx = (uint16_t*)(blob + L.rowidx);
+    int32_t* c2r = (int32_t*)(blob + L.c2r);
+    unsigned long long* put = (unsigned long long*)(blob + L.rowval);  // (column, entry) of a row, unordered
+    for (int pos = tid; pos < n; pos += BT) {
+      const int t = W.posnode[pos];
+      gidx[pos] = pc_of_local(se, A.elem_ptr, t);
+      perm[pos] = (uint16_t)t;
+    }
+    for (int q = tid; q <= nlev; q += BT) lvl[q] = (uint16_t)W.lvl[q];
+    for (int q = tid; q <= n; q += BT) {
+      colptr[q] = (uint32_t)W.colstart[q];
+      rowptr[q] = (uint32_t)W.rstart[q];
+    }
+    for (int q = tid; q < ncol; q += BT) colidx[q] = W.colent[q];
+    // row form: the entries of each row in any order, then by column (every row lists its
+    // columns ascending)
+    for (int v = wid; v < n; v += BT / 32)
+      for (int q = W.colstart[v] + lane; q < W.colstart[v + 1]; q += 32) {
+        const int i = W.colent[q];
+        put[W.rstart[i] + atomicAdd(&W.rcnt[i], 1)] = ((unsigned long long)v << 32) | (unsigned)q;
+      }
+    __syncthreads();
+    for (int i = wid; i < n; i += BT / 32) {
+      const int r0 = W.rstart[i], r1 = W.rstart[i + 1];
+      for (int q = r0 + lane; q < r1; q += 32) {
+        const unsigned long long e = put[q];
+        int rank = 0;
+        for (int p = r0; p < r1; ++p) rank += put[p] < e;
+        rowidx[r0 + rank] = (uint16_t)(e >> 32);
+        c2r[(unsigned)e] = r0 + rank;
+      }
+    }
+    __syncthreads();
+  }
+}
+
 // the longest row of K (entries), for the adjacency capacity
 __global__ void k_max_row(int64_t n, const int64_t* __restrict__ ptr, int* out) {
   int m = 0;
@@ -803,19 +1168,23 @@ static int factor_stars(spnet_pc_s* pc, int32_t* noinv, int* ill) {
   }
   const int acap = adjacency_cap(max_row - 1, pc->d, pc->max_star);
   const int64_t hot = hot_bytes(nmax, acap);
-  // hot arrays in shared memory when four warps' worth fit in 200 KiB, one
-  // block of four warps per SM at least; otherwise everything in global scratch
-  const int hot_in_smem = 4 * hot <= 200 * 1024 ? 1 : 0;
-  int wpb_blocks = hot_in_smem ? (int)((200 * 1024) / (4 * hot)) : 4;  // blocks per SM
-  if (wpb_blocks < 1) wpb_blocks = 1;
-  if (wpb_blocks > 4) wpb_blocks = 4;
-  if (hot_in_smem) {
+  // a warp per star with everything in shared memory when four warps' worth fit in 200 KiB,
+  // else a block of four warps per star (its marks in shared memory while they fit)
+  const bool per_warp = 4 * hot <= 200 * 1024;
+  const int64_t marks = (BT / 32) * bitmap_bytes(nmax) + marks_bytes(nmax);
+  const int hot_in_smem = per_warp || marks <= 200 * 1024 ? 1 : 0;
+  const size_t smem = per_warp ? (size_t)(4 * hot)
+                               : (size_t)(hot_in_smem ? marks : (BT / 32) * bitmap_bytes(nmax));
+  int per_sm = (int)((200 * 1024) / (smem + 1024));  // blocks per SM
+  per_sm = per_sm < 1 ? 1 : per_sm > (per_warp ? 4 : 8) ? (per_warp ? 4 : 8) : per_sm;
+  {
     static std::atomic<bool> attr_set[64];  // per device
     int dev = 0;
     SPNET_CUDA_TRY(cudaGetDevice(&dev));
     dev &= 63;
     if (!attr_set[dev]) {
       SPNET_CUDA_TRY(cudaFuncSetAttribute(k_star_symbolic, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
+      SPNET_CUDA_TRY(cudaFuncSetAttribute(k_star_symbolic_block, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
       attr_set[dev] = true;
     }
   }
@@ -828,19 +1197,19 @@ static int factor_stars(spnet_pc_s* pc, int32_t* noinv, int* ill) {
   int core_max = core_inv > 0 ? 0
                  : nmax <= 4 * CORE_FIRST ? (nmax < CORE_FIRST ? nmax : CORE_FIRST)
                                           : 4 * CORE_FIRST;
-  int64_t stride = 0, warps = 0;
+  int64_t stride = 0, workers = 0;  // scratch of a worker (a warp or a block)
   char* scratch = nullptr;
   auto size_scratch = [&]() -> int {
-    stride = cold_bytes(nmax, core_max, acap) + (hot_in_smem ? 0 : align_up(hot, 256));
-    warps = (int64_t)4 * wpb_blocks * num_sms();
+    stride = cold_bytes(nmax, core_max, acap) + (per_warp ? 0 : align_up(hot, 256));
+    workers = (int64_t)(per_warp ? 4 : 1) * per_sm * num_sms();
     const int64_t budget = (int64_t)1 << 30;
-    if (warps * stride > budget) warps = budget / stride;
-    if (warps < 4) warps = 4;
-    if (warps > pc->S) warps = pc->S;
-    warps = (warps + 3) / 4 * 4;
+    if (workers * stride > budget) workers = budget / stride;
+    if (workers > pc->S) workers = pc->S;
+    if (workers < 1) workers = 1;
+    if (per_warp) workers = (workers + 3) / 4 * 4;
     if (scratch) tmp.release(scratch);
     scratch = nullptr;
-    return tmp.get(&scratch, warps * stride);
+    return tmp.get(&scratch, workers * stride);
   };
   SPNET_TRY(size_scratch());
   int* counters = nullptr;  // [0] next star, [2..3] pool top (u64)
@@ -892,7 +1261,8 @@ static int factor_stars(spnet_pc_s* pc, int32_t* noinv, int* ill) {
     A.N = pc->N;
     note_launch();
     ProfScope ps(KID_STAR_SYMBOLIC, s);
-    k_star_symbolic<<<(unsigned)(warps / 4), 128, hot_in_smem ? (size_t)(4 * hot) : 0, s>>>(A);
+    if (per_warp) k_star_symbolic<<<(unsigned)(workers / 4), 128, smem, s>>>(A);
+    else k_star_symbolic_block<<<(unsigned)workers, BT, smem, s>>>(A);
     SPNET_CUDA_TRY(cudaGetLastError());
     int h = 0;
     SPNET_CUDA_TRY(cudaMemcpyAsync(&h, flags, sizeof(int), cudaMemcpyDeviceToHost, s));
