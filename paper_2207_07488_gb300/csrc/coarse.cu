@@ -781,8 +781,21 @@ __global__ void __launch_bounds__(256) k_coarse_batch(const T* __restrict__ tile
   int I, J;
   upper_tile(blockIdx.x, nt, &I, &J);
   const T* Zt = tiles + (int64_t)blockIdx.x * CT * CT;
-  for (int q = threadIdx.x; q < CT * CT; q += blockDim.x) Zs[q / CT][q % CT] = Zt[q];
+  // 16 bytes a load (32 in FP64), eight in flight: the tile is most of what a block waits for
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    Vec4<T> v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) v[u] = load4(Zt + 4 * ((h * 8 + u) * 256 + (int)threadIdx.x));
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int q = 4 * ((h * 8 + u) * 256 + (int)threadIdx.x);
+#pragma unroll
+      for (int e = 0; e < 4; ++e) Zs[q / CT][q % CT + e] = v[u].v[e];
+    }
+  }
   // the restricted right-hand sides of the tile's row and column blocks
+#pragma unroll 8
   for (int q = threadIdx.x; q < 2 * CT * KP; q += blockDim.x) {
     const int side = q / (CT * KP), u = (q / KP) % CT, j = q % KP;
     const int64_t ci = (int64_t)(side == 0 ? I : J) * CT + u;
@@ -811,9 +824,15 @@ __global__ void __launch_bounds__(256) k_coarse_batch(const T* __restrict__ tile
     }
     T* out = part + ((int64_t)I * nt + J) * CT * KP;
 #pragma unroll
-    for (int a = 0; a < BT::UR; ++a)
+    for (int a = 0; a < BT::UR; ++a) {
+      T* o = out + (ut + a * BT::TPG) * KP + j0;
+      if constexpr (BT::JR == 4) {
+        st4(o, acc[a]);
+      } else {
 #pragma unroll
-      for (int b = 0; b < BT::JR; ++b) out[(ut + a * BT::TPG) * KP + j0 + b] = acc[a][b];
+        for (int b = 0; b < BT::JR; ++b) o[b] = acc[a][b];
+      }
+    }
   }
   if (I != J) {  // part[J][I][c][j] = sum_u Z[u][c] R_I[u][j]
     T acc[BT::UR][BT::JR];
@@ -834,9 +853,15 @@ __global__ void __launch_bounds__(256) k_coarse_batch(const T* __restrict__ tile
     }
     T* out = part + ((int64_t)J * nt + I) * CT * KP;
 #pragma unroll
-    for (int a = 0; a < BT::UR; ++a)
+    for (int a = 0; a < BT::UR; ++a) {
+      T* o = out + (ut + a * BT::TPG) * KP + j0;
+      if constexpr (BT::JR == 4) {
+        st4(o, acc[a]);
+      } else {
 #pragma unroll
-      for (int b = 0; b < BT::JR; ++b) out[(ut + a * BT::TPG) * KP + j0 + b] = acc[a][b];
+        for (int b = 0; b < BT::JR; ++b) o[b] = acc[a][b];
+      }
+    }
   }
 }
 
