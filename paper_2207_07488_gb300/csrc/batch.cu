@@ -59,12 +59,35 @@ __device__ __forceinline__ void column_partials(double v, int kp, double* part, 
   __syncthreads();
 }
 
-// sum over nb blocks of column j's partials (by one warp; every lane gets it); fixed order
-__device__ __forceinline__ double column_total(const double* part, int nb, int j) {
-  double t = 0.0;
-  for (int b = threadIdx.x & 31; b < nb; b += 32) t += __ldcg(&part[(int64_t)b * KMAX + j]);
-  for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-  return t;
+// Sums over the blocks of NS sets of column partials ([blocks][KMAX] each), by a block of 256
+// threads: warp w adds the rows b = w, w + 8, .. of every set, lane = column (a row is 256
+// contiguous bytes), eight loads in flight; the warps' sums are added in order.  out[s][j] in
+// shared memory.  The last block runs alone, so its loads are all there is: a warp per column
+// with strided loads took 10-15 us of the combine on the 3D workload with 32 right-hand sides.
+template <int NS>
+__device__ void column_totals(const double* const (&part)[NS], const int (&nb)[NS], double (*sh)[8][KMAX],
+                              double (*out)[KMAX]) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+#pragma unroll
+  for (int s = 0; s < NS; ++s) {
+    double t = 0.0;
+    for (int b0 = wid; b0 < nb[s]; b0 += 64) {
+      double v[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) v[u] = b0 + 8 * u < nb[s] ? __ldcg(&part[s][(int64_t)(b0 + 8 * u) * KMAX + lane]) : 0.0;
+#pragma unroll
+      for (int u = 0; u < 8; ++u) t += v[u];
+    }
+    sh[s][wid][lane] = t;
+  }
+  __syncthreads();
+  if (wid < NS) {
+    double t = sh[wid][0][lane];
+#pragma unroll
+    for (int w = 1; w < 8; ++w) t += sh[wid][w][lane];
+    out[wid][lane] = t;
+  }
+  __syncthreads();
 }
 
 // P = Z + beta P, Q = A Z + beta Q per column; partials of (p_j, q_j); last block: alpha_j
@@ -98,24 +121,29 @@ __global__ void __launch_bounds__(256) k_bspmm_dir(int64_t n, int k, int kp, con
   }
   column_partials(dot, kp, part, sh);
   if (last_block(&bs->cnt[0])) {
-    for (int jj = threadIdx.x >> 5; jj < k; jj += (int)(blockDim.x >> 5)) {
-      const double pq = column_total(part, gridDim.x, jj);
-      if ((threadIdx.x & 31) == 0) {
-        bs->pq[jj] = pq;
-        bs->alpha[jj] = (bs->done[jj] || pq == 0.0) ? 0.0 : bs->rz[jj] / pq;
-      }
+    __shared__ double tsh[1][8][KMAX], tot[1][KMAX];
+    const double* const ps[1] = {part};
+    const int nb[1] = {(int)gridDim.x};
+    column_totals<1>(ps, nb, tsh, tot);
+    if ((int)threadIdx.x < k) {
+      const int jj = threadIdx.x;
+      const double pq = tot[0][jj];
+      bs->pq[jj] = pq;
+      bs->alpha[jj] = (bs->done[jj] || pq == 0.0) ? 0.0 : bs->rz[jj] / pq;
     }
     if (threadIdx.x == 0) bs->cnt[0] = 0;
   }
 }
 
-// one warp per element, lanes (row r, column j); mode 0: X += alpha P, R -= alpha Q;
-// mode 1: R as is.  Partials of |r_j|^2; corner sums EP[(e, corner, comp)][j] of
-// phi_c r_j.  A lane takes BU of the element's dofs at a time, every load first.
+// A team of `team` warps per element, lanes (row r, column j); mode 0: X += alpha P, R -= alpha
+// Q; mode 1: R as is.  Partials of |r_j|^2; corner sums EP[(e, corner, comp)][j] of phi_c r_j.
+// A lane takes BU of the element's dofs at a time, every load first.  With one dof per node the
+// warps' corner sums meet in shared memory (in order); a warp per element left 27 warps on an
+// SM with 40 dofs each to walk (80 us a launch on the 3D workload with 32 right-hand sides).
 constexpr int BU = 4;
 
 template <int NC, int ND, class CT>
-__global__ void __launch_bounds__(256) k_bupdate(int n_elem, int64_t N, int k, int kp,
+__global__ void __launch_bounds__(256) k_bupdate(int n_elem, int64_t N, int k, int kp, int team,
                                                  const int32_t* __restrict__ elem_ptr,
                                                  const int8_t* __restrict__ comp_of, const CT* __restrict__ xi,
                                                  double* __restrict__ X, double* __restrict__ R,
@@ -124,23 +152,24 @@ __global__ void __launch_bounds__(256) k_bupdate(int n_elem, int64_t N, int k, i
                                                  int simplex) {
   constexpr int D = NC == 4 ? 2 : 3;
   __shared__ double sh[8][KMAX];
+  __shared__ CT corner[ND == 1 ? 8 : 1][ND == 1 ? NC : 1][KMAX];
   pdl_wait();
   pdl_trigger();
   if (mode == 0 && bs->all_done) return;
-  const int lane = threadIdx.x & 31;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int rows = 32 / kp, r = lane / kp, j = lane % kp;
   const bool act = j < k;
   const double alpha = (mode == 0 && act) ? bs->alpha[j] : 0.0;
-  const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  const int per = 8 / team, tw = wid % team;  // elements a block takes at a time; this warp's place
   double rr = 0.0;
-  for (int64_t e = gw; e < n_elem; e += nw) {
+  for (int64_t e0 = (int64_t)blockIdx.x * per; e0 < n_elem; e0 += (int64_t)gridDim.x * per) {
+    const int64_t e = e0 + wid / team;
     CT acc[NC * ND];
 #pragma unroll
     for (int t = 0; t < NC * ND; ++t) acc[t] = CT(0);
-    const int a0 = elem_ptr[e], a1 = elem_ptr[e + 1];
+    const int a0 = e < n_elem ? elem_ptr[e] : 0, a1 = e < n_elem ? elem_ptr[e + 1] : 0;
     if (act) {
-      for (int i0 = a0 + r; i0 < a1; i0 += rows * BU) {
+      for (int i0 = a0 + tw * rows * BU + r; i0 < a1; i0 += team * rows * BU) {
         bool ok[BU];
         int ii[BU], cm[BU];
         double xv[BU], pv[BU], qv[BU], rv[BU];
@@ -188,17 +217,31 @@ __global__ void __launch_bounds__(256) k_bupdate(int n_elem, int64_t N, int k, i
     for (int t = 0; t < NC * ND; ++t) {
       CT v = acc[t];
       for (int o = kp; o < 32; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-      if (r == 0 && act) EP[(e * (NC * ND) + t) * k + j] = (double)v;
+      if (ND == 1) corner[wid][t % (ND == 1 ? NC : 1)][lane] = v;
+      else if (r == 0 && act && e < n_elem) EP[(e * (NC * ND) + t) * k + j] = (double)v;
+    }
+    if (ND == 1) {
+      __syncthreads();
+      // (element, corner, column): the team's sums in order
+      for (int q = threadIdx.x; q < per * NC * KMAX; q += 256) {
+        const int el = q / (NC * KMAX), t = q / KMAX % NC, jj = q % KMAX;
+        if (jj < k && e0 + el < n_elem) {
+          CT v = corner[el * team][t][jj];
+          for (int w = 1; w < team; ++w) v += corner[el * team + w][t][jj];
+          EP[((e0 + el) * NC + t) * k + jj] = (double)v;
+        }
+      }
+      __syncthreads();
     }
   }
   column_partials(rr, kp, part, sh);
 }
 
-// one warp per element: Z = R_0^T Z_c + sum_j E_j W_j per column; with dots,
+// `team` warps per element: Z = R_0^T Z_c + sum_j E_j W_j per column; with dots,
 // partials of (r_j, z_j), (r_j, z_old_j) and in the last block beta_j, |r_j|^2
 // (from the update's partials), the stop tests (dots 1: a PCG step; 2: the start)
 template <int NC, int ND, class CT, class WS>
-__global__ void __launch_bounds__(256) k_bcombine(int n_elem, int64_t N, int k, int kp,
+__global__ void __launch_bounds__(256) k_bcombine(int n_elem, int64_t N, int k, int kp, int team,
                                                   const int32_t* __restrict__ elem_ptr,
                                                   const int8_t* __restrict__ comp_of, const CT* __restrict__ xi,
                                                   const int32_t* __restrict__ ecoarse,
@@ -218,8 +261,10 @@ __global__ void __launch_bounds__(256) k_bcombine(int n_elem, int64_t N, int k, 
   const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
   double s1 = 0.0, s2 = 0.0;
-  for (int64_t e = gw; e < n_elem; e += nw) {
+  for (int64_t it = gw; it < (int64_t)n_elem * team; it += nw) {
     if (!act) continue;
+    const int64_t e = it / team;
+    const int tw = (int)(it - e * team);
     CT zcv[NC * ND];
 #pragma unroll
     for (int t = 0; t < NC * ND; ++t) {
@@ -234,7 +279,7 @@ __global__ void __launch_bounds__(256) k_bcombine(int n_elem, int64_t N, int k, 
 #pragma unroll
     for (int c = 0; c < NC; ++c) sb[c] = with_stars ? (int)estar[e * NC + c] : -1;
     const int a0 = elem_ptr[e], a1 = elem_ptr[e + 1];
-    for (int i0 = a0 + r; i0 < a1; i0 += rows * BU) {
+    for (int i0 = a0 + tw * rows * BU + r; i0 < a1; i0 += team * rows * BU) {
       bool ok[BU];
       int ii[BU], cm[BU];
       CT t[BU][3], wv[BU][NC];
@@ -282,22 +327,23 @@ __global__ void __launch_bounds__(256) k_bcombine(int n_elem, int64_t N, int k, 
   column_partials(s1, kp, part1, sh);
   column_partials(s2, kp, part2, sh);
   if (last_block(&bs->cnt[2])) {
-    for (int jj = threadIdx.x >> 5; jj < k; jj += (int)(blockDim.x >> 5)) {
-      const double rz_new = column_total(part1, gridDim.x, jj);
-      const double rzo = column_total(part2, gridDim.x, jj);
-      const double rr = dots == 1 ? column_total(prr, nrr, jj) : 0.0;
-      if ((threadIdx.x & 31) == 0) {
-        if (dots == 2) {  // PCG start: beta = 0
-          bs->beta[jj] = 0.0;
-          bs->rz[jj] = rz_new;
-        } else if (!bs->done[jj]) {
-          const double rz = bs->rz[jj];
-          bs->beta[jj] = rz == 0.0 ? 0.0 : (flexible ? (rz_new - rzo) / rz : rz_new / rz);
-          bs->rz[jj] = rz_new;
-          bs->rr[jj] = rr;
-          bs->iters[jj] = bs->iter + 1;
-          if (sqrt(rr) <= bs->rtol * sqrt(bs->bb[jj]) || bs->iter + 1 >= bs->maxit) bs->done[jj] = 1;
-        }
+    __shared__ double tsh[3][8][KMAX], tot[3][KMAX];
+    const double* const ps[3] = {part1, part2, prr};
+    const int nb[3] = {(int)gridDim.x, (int)gridDim.x, dots == 1 ? nrr : 0};
+    column_totals<3>(ps, nb, tsh, tot);
+    if ((int)threadIdx.x < k) {
+      const int jj = threadIdx.x;
+      const double rz_new = tot[0][jj], rzo = tot[1][jj], rr = tot[2][jj];
+      if (dots == 2) {  // PCG start: beta = 0
+        bs->beta[jj] = 0.0;
+        bs->rz[jj] = rz_new;
+      } else if (!bs->done[jj]) {
+        const double rz = bs->rz[jj];
+        bs->beta[jj] = rz == 0.0 ? 0.0 : (flexible ? (rz_new - rzo) / rz : rz_new / rz);
+        bs->rz[jj] = rz_new;
+        bs->rr[jj] = rr;
+        bs->iters[jj] = bs->iter + 1;
+        if (sqrt(rr) <= bs->rtol * sqrt(bs->bb[jj]) || bs->iter + 1 >= bs->maxit) bs->done[jj] = 1;
       }
     }
     __syncthreads();
@@ -378,15 +424,30 @@ static int batch_alloc(spnet_pc_s* pc, Batch& b, int k, DevArena& tmp, bool iter
   return SPNET_OK;
 }
 
-// blocks of 8 warps, one element per warp, at most PG (the stride of the partial slots)
-static int elem_blocks(const spnet_pc_s* pc) {
-  const int need = (pc->n_elem + 7) / 8;
-  return need < 1 ? 1 : need > pc->PG ? pc->PG : need;
+// Warps per element: doubled while each keeps at least `keep` batches (of 32 / kp * BU dofs) to
+// walk.  Measured, us a launch: 3D workload, 32 right-hand sides (10 batches an element): update
+// 83 with one warp, 74 with two, 74 with four; combine (whose warps each load the element's
+// coarse values) 126, 132, 175.  2D, 290 dofs an element, 7 right-hand sides (18 batches):
+// update 77, 50, 43, 42 with eight; combine 99, 71, 73, 90.  3D, 61 dofs, 3 right-hand sides (2
+// batches): update 15.5, 17.4; combine 27, 34.
+static int elem_team(const spnet_pc_s* pc, int kp, int keep, int most) {
+  const int64_t avg = pc->n_elem > 0 ? (pc->N + pc->n_elem - 1) / pc->n_elem : 1;
+  const int64_t batches = avg * kp / (32 * BU);
+  int t = 1;
+  while (t < most && t * 2 * keep <= batches) t *= 2;
+  return t;
+}
+static int update_team(const spnet_pc_s* pc, int kp) { return pc->ndof == 1 ? elem_team(pc, kp, 4, 8) : 1; }
+static int combine_team(const spnet_pc_s* pc, int kp) { return elem_team(pc, kp, 8, 8); }
+static int elem_blocks(const spnet_pc_s* pc, int team) {
+  const int64_t need = ((int64_t)pc->n_elem * team + 7) / 8;
+  return need < 1 ? 1 : need > pc->PG ? pc->PG : (int)need;
 }
 
 template <int NC, int ND, class CT>
 static void bupdate_t(spnet_pc_s* pc, Batch& b, const CT* xi, int mode, cudaStream_t s) {
-  launch_pdl(k_bupdate<NC, ND, CT>, elem_blocks(pc), 256, 0, s, pc->n_elem, pc->N, b.k, b.kp,
+  const int team = update_team(pc, b.kp);
+  launch_pdl(k_bupdate<NC, ND, CT>, elem_blocks(pc, team), 256, 0, s, pc->n_elem, pc->N, b.k, b.kp, team,
              (const int32_t*)pc->elem_ptr, (const int8_t*)pc->comp_of, xi, b.X, b.R, (const double*)b.P,
              (const double*)b.Q, b.EP, b.p1, b.bs, mode, pc->coarse_space == SPNET_COARSE_P1 ? 1 : 0);
 }
@@ -408,10 +469,11 @@ static void launch_bupdate(spnet_pc_s* pc, Batch& b, int mode, cudaStream_t s) {
 
 template <int NC, int ND, class CT, class WS>
 static void bcombine_t(spnet_pc_s* pc, Batch& b, const CT* xi, int wc, int ws, int dots, cudaStream_t s) {
-  launch_pdl(k_bcombine<NC, ND, CT, WS>, elem_blocks(pc), 256, 0, s, pc->n_elem, pc->N, b.k, b.kp,
+  const int team = combine_team(pc, b.kp);
+  launch_pdl(k_bcombine<NC, ND, CT, WS>, elem_blocks(pc, team), 256, 0, s, pc->n_elem, pc->N, b.k, b.kp, team,
              (const int32_t*)pc->elem_ptr, (const int8_t*)pc->comp_of, xi, (const int32_t*)pc->ecoarse,
              (const int64_t*)pc->estar, (const double*)b.ZC, (const WS*)b.W, (const double*)b.R, b.Z, b.p2, b.p3,
-             (const double*)b.p1, elem_blocks(pc), (int)(wc && pc->m0 > 0), (int)(ws && pc->S > 0), b.bs, dots,
+             (const double*)b.p1, elem_blocks(pc, update_team(pc, b.kp)), (int)(wc && pc->m0 > 0), (int)(ws && pc->S > 0), b.bs, dots,
              pc->flexible, pc->coarse_space == SPNET_COARSE_P1 ? 1 : 0);
 }
 
