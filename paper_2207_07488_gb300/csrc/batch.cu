@@ -603,6 +603,11 @@ int pcg_batch_run(spnet_op_s* op, spnet_pc_s* pc, int k, const double* df, const
   h.k = k;
   h.maxit = maxit;
   unsigned* cnt3 = &pc->scal->cnt[3];
+  // the scalars of each right-hand side are kept on the device and read back together: a wait
+  // for each one left the GPU idle between them
+  Scal* dsc = nullptr;
+  SPNET_TRY(tmp.get(&dsc, k));
+  std::vector<Scal> hsc(k);
   for (int j = 0; j < k; ++j) {
     note_launch();
     k_build_rhs<<<G, 256, 0, s>>>(N, pc->perm, op->free_dofs, df + (int64_t)j * nd, op->fd.ptr, op->fd.col,
@@ -623,9 +628,12 @@ int pcg_batch_run(spnet_op_s* op, spnet_pc_s* pc, int k, const double* df, const
     k_col_put<<<G, 256, 0, s>>>(N, k, j, pc->x, b.X);
     note_launch();
     k_col_put<<<G, 256, 0, s>>>(N, k, j, pc->r, b.R);
-    Scal sc{};
-    SPNET_CUDA_TRY(cudaMemcpyAsync(&sc, pc->scal, sizeof(Scal), cudaMemcpyDeviceToHost, s));
-    SPNET_CUDA_TRY(cudaStreamSynchronize(s));
+    SPNET_CUDA_TRY(cudaMemcpyAsync(dsc + j, pc->scal, sizeof(Scal), cudaMemcpyDeviceToDevice, s));
+  }
+  SPNET_CUDA_TRY(cudaMemcpyAsync(hsc.data(), dsc, sizeof(Scal) * k, cudaMemcpyDeviceToHost, s));
+  SPNET_CUDA_TRY(cudaStreamSynchronize(s));
+  for (int j = 0; j < k; ++j) {
+    const Scal& sc = hsc[j];
     if (!std::isfinite(sc.bb) || !std::isfinite(sc.rr)) {  // (the guard releases the events)
       return fail(SPNET_ERR_BAD_INPUT, std::isfinite(sc.bb)
                                            ? "pcg_solve: non-finite initial guess"
@@ -698,9 +706,13 @@ int pcg_batch_run(spnet_op_s* op, spnet_pc_s* pc, int k, const double* df, const
     k_residual<<<G, 256, 0, s>>>(N, pc->b, pc->q, pc->vtmp, pc->partial, &pc->scal->rr_true, cnt3);
     note_launch();
     k_expand<<<G, 256, 0, s>>>(nd, op->free_of, pc->iperm, pc->x, dg + (int64_t)j * ndir, xj);
-    Scal sc{};
-    SPNET_CUDA_TRY(cudaMemcpyAsync(&sc, pc->scal, sizeof(Scal), cudaMemcpyDeviceToHost, s));
-    SPNET_CUDA_TRY(cudaStreamSynchronize(s));
+    SPNET_CUDA_TRY(cudaMemcpyAsync(dsc + j, pc->scal, sizeof(Scal), cudaMemcpyDeviceToDevice, s));
+  }
+  SPNET_CUDA_TRY(cudaMemcpyAsync(hsc.data(), dsc, sizeof(Scal) * k, cudaMemcpyDeviceToHost, s));
+  SPNET_CUDA_TRY(cudaStreamSynchronize(s));
+  for (int j = 0; j < k; ++j) {
+    double* xj = dx + (int64_t)j * nd;
+    const Scal& sc = hsc[j];
     const double rel = h.bb[j] > 0.0 ? sqrt(sc.rr_true) / sqrt(h.bb[j]) : 0.0;
     spnet_stats st{};
     st.iterations = h.iters[j];
