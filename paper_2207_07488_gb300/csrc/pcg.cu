@@ -262,7 +262,7 @@ __global__ void __launch_bounds__(128, ND == 1 ? 7 : 4) k_combine(int n_elem, in
                                                  int nrr, int with_coarse, int with_stars, Scal* sc,
                                                  int flexible, int first, int simplex) {
   constexpr int D = NC == 4 ? 2 : 3;
-  __shared__ double sh[64];
+  __shared__ double sh[32];
   pdl_wait();
   pdl_trigger();
   if (sc && sc->done) return;
@@ -326,7 +326,8 @@ __global__ void __launch_bounds__(128, ND == 1 ? 7 : 4) k_combine(int n_elem, in
     }
   }
   if (!sc) return;
-  block_partial2(s1, s2, part1, part2, sh);
+  block_partial(s1, part1, sh);
+  block_partial(s2, part2, sh);
   if (last_block(&sc->cnt[2])) {
     // in a PCG step also |r|^2 of the update, the iteration count and the stop test
     __shared__ double sh3[96];

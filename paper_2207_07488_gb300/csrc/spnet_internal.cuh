@@ -545,42 +545,14 @@ __device__ __forceinline__ void block_partial(double v, double* out, double* sh)
   __syncthreads();
 }
 
-// two such sums at once (sh: 64 doubles)
-__device__ __forceinline__ void block_partial2(double v0, double v1, double* out0, double* out1, double* sh) {
-  for (int o = 16; o > 0; o >>= 1) {
-    v0 += __shfl_xor_sync(0xffffffffu, v0, o);
-    v1 += __shfl_xor_sync(0xffffffffu, v1, o);
-  }
-  if ((threadIdx.x & 31) == 0) {
-    sh[threadIdx.x >> 5] = v0;
-    sh[32 + (threadIdx.x >> 5)] = v1;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double t0 = 0.0, t1 = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
-      t0 += sh[w];
-      t1 += sh[32 + w];
-    }
-    out0[blockIdx.x] = t0;
-    out1[blockIdx.x] = t1;
-  }
-  __syncthreads();
-}
-
-// true in the block that finishes last (its partials and everyone's are visible).  Only one
-// thread fences: the barrier before it orders the block's partials ahead of its fence, and
-// nothing else a block writes is read before the kernel ends (a fence in every thread waits
-// for all of the block's stores).
+// true in the block that finishes last (its partials and everyone's are visible)
 __device__ __forceinline__ bool last_block(unsigned* cnt) {
   __shared__ bool is_last;
+  __threadfence();
   __syncthreads();
-  if (threadIdx.x == 0) {
-    __threadfence();
-    is_last = atomicAdd(cnt, 1u) == gridDim.x - 1;
-    __threadfence();
-  }
+  if (threadIdx.x == 0) is_last = atomicAdd(cnt, 1u) == gridDim.x - 1;
   __syncthreads();
+  if (is_last) __threadfence();
   return is_last;
 }
 
