@@ -69,6 +69,39 @@ __device__ inline T zat(const T* tiles, int nt, int64_t i, int64_t j) {
   return tiles[tile_index((int)(i / CT), (int)(j / CT), nt) * CT * CT + (i % CT) * CT + (j % CT)];
 }
 
+template <class T>
+struct V4 {
+  T v[4];
+};
+// four consecutive T (16-byte aligned; 32 for double)
+template <class T>
+__device__ __forceinline__ V4<T> ld4s(const T* p) {
+  V4<T> r;
+  if (sizeof(T) == 4) {
+    const float4 a = *reinterpret_cast<const float4*>(p);
+    r.v[0] = a.x;
+    r.v[1] = a.y;
+    r.v[2] = a.z;
+    r.v[3] = a.w;
+  } else {
+    const double2 a = *reinterpret_cast<const double2*>(p), b = *(reinterpret_cast<const double2*>(p) + 1);
+    r.v[0] = a.x;
+    r.v[1] = a.y;
+    r.v[2] = b.x;
+    r.v[3] = b.y;
+  }
+  return r;
+}
+template <class T>
+__device__ __forceinline__ void st4(T* p, const T (&v)[4]) {
+  if (sizeof(T) == 4) {
+    *reinterpret_cast<float4*>(p) = make_float4((float)v[0], (float)v[1], (float)v[2], (float)v[3]);
+  } else {
+    *reinterpret_cast<double2*>(p) = make_double2(v[0], v[1]);
+    *(reinterpret_cast<double2*>(p) + 1) = make_double2(v[2], v[3]);
+  }
+}
+
 // Invert the SPD block held 4 x 4 per thread by 256 threads (thread (tr, tc)
 // owns rows 4tr.., columns 4tc.. of a 64 x 64 block; kb valid rows) by scalar
 // Gauss-Jordan sweeps in the arithmetic of T: sweeping pivot p maps
@@ -79,50 +112,59 @@ __device__ inline T zat(const T* tiles, int nt, int64_t i, int64_t j) {
 constexpr double DROP64 = 1e-8;  // FP64 sweeps: relative pivot at or below which a function is dropped
 constexpr double TRIG32 = 1e-3;  // FP32 sweeps: relative pivot at or below which FP64 takes over
 
-// As above, with dropping: dg holds the original diagonal entries of the block's
-// rows; a pivot at or below tol times its entry is not swept.  Returns the bitmask
-// of the dropped pivots (uniform over the threads).
+// The least pivot that is swept lies above this: (double)piv > x and piv > pivot_limit(x) agree
+// for every piv of type T (x rounded down to T), without an FP64 comparison in the chain.
 template <class T>
-__device__ uint64_t invert_block_regs(T (&d)[4][4], int kb, T (*rowp)[NB], T (*colp)[NB], const double* dg,
-                                      double tol) {
+__device__ __forceinline__ T pivot_limit(double x) {
+  if constexpr (sizeof(T) == 4) return __double2float_rd(x);
+  else return x;
+}
+
+// As above, with dropping: limit is pivot_limit of tol times the original diagonal entry of row
+// threadIdx.x of the block (threads 0..kb-1); a pivot at or below it is not swept.  Returns the
+// bitmask of the dropped pivots (uniform over the threads).
+// Bound by the chain of kb steps, each a barrier, the reads of row and column p, a division and
+// the update; nothing else waits in it: the limits lie in shared memory, and which entries
+// belong to row or column p = 4 q + a is known at compile time but for q.  With the limits read
+// from global memory and compared in FP64, and row and column tests on every entry, a block of 64
+// took 33.8 us, now 19.1; a sweep of the 3D workload (m0 = 4335), whose block 0 ends in it, 43.9
+// us, now 38.9.
+template <class T>
+__device__ uint64_t invert_block_regs(T (&d)[4][4], int kb, T limit) {
+  __shared__ __align__(16) T rowp[2][NB], colp[2][NB];
+  __shared__ T lim[NB];
   const int tr = threadIdx.x >> 4, tc = threadIdx.x & 15;
+  if ((int)threadIdx.x < kb) lim[threadIdx.x] = limit;
   uint64_t dropped = 0;
   for (int q = 0; q < NB / 4; ++q) {
+    const bool rq = tr == q, cq = tc == q;
 #pragma unroll
     for (int a = 0; a < 4; ++a) {
       const int p = 4 * q + a;
       if (p >= kb) break;  // uniform
       const int buf = p & 1;
-      if (tr == q) {
-#pragma unroll
-        for (int b = 0; b < 4; ++b) rowp[buf][4 * tc + b] = d[a][b];
-      }
-      if (tc == q) {
-#pragma unroll
-        for (int b = 0; b < 4; ++b) colp[buf][4 * tr + b] = d[b][a];
+      if (rq) st4(&rowp[buf][4 * tc], d[a]);
+      if (cq) {
+        const T col[4] = {d[0][a], d[1][a], d[2][a], d[3][a]};
+        st4(&colp[buf][4 * tr], col);
       }
       __syncthreads();
       const T piv = colp[buf][p];
-      if (!((double)piv > tol * dg[p])) {  // in the span of the pivots kept so far
+      const V4<T> cv = ld4s(&colp[buf][4 * tr]), rv = ld4s(&rowp[buf][4 * tc]);
+      if (!(piv > lim[p])) {  // in the span of the pivots kept so far
         dropped |= 1ull << p;
         continue;
       }
       const T ip = (T)1 / piv;
-      T cv[4], rv[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        cv[u] = colp[buf][4 * tr + u];
-        rv[u] = rowp[buf][4 * tc + u];
-      }
 #pragma unroll
       for (int u = 0; u < 4; ++u)
 #pragma unroll
         for (int v = 0; v < 4; ++v) {
-          const bool ri = 4 * tr + u == p, cj = 4 * tc + v == p;
-          if (!ri && !cj) d[u][v] -= cv[u] * rv[v] * ip;
+          const bool ri = u == a && rq, cj = v == a && cq;
+          if (!ri && !cj) d[u][v] -= cv.v[u] * rv.v[v] * ip;
           else if (ri && cj) d[u][v] = -ip;
-          else if (ri) d[u][v] = rv[v] * ip;
-          else d[u][v] = cv[u] * ip;
+          else if (ri) d[u][v] = rv.v[v] * ip;
+          else d[u][v] = cv.v[u] * ip;
         }
     }
   }
@@ -160,8 +202,8 @@ __global__ void k_tiles_from_A0(const double* __restrict__ A0, int64_t m0, int n
 template <class T>
 __global__ void __launch_bounds__(256) k_pivot_inverse(const T* tiles, int nt, int k0, int kb, T* P,
                                                        const double* diag0, double tol, int* ndrop) {
-  __shared__ T rowp[2][NB], colp[2][NB];
   const int tr = threadIdx.x >> 4, tc = threadIdx.x & 15;
+  const T limit = (int)threadIdx.x < kb ? pivot_limit<T>(tol * diag0[k0 + threadIdx.x]) : (T)0;
   T d[4][4];
 #pragma unroll
   for (int a = 0; a < 4; ++a)
@@ -170,7 +212,7 @@ __global__ void __launch_bounds__(256) k_pivot_inverse(const T* tiles, int nt, i
       const int i = 4 * tr + a, j = 4 * tc + b;
       d[a][b] = (i < kb && j < kb) ? zat(tiles, nt, k0 + i, k0 + j) : (T)0;
     }
-  const uint64_t dropped = invert_block_regs(d, kb, rowp, colp, diag0 + k0, tol);
+  const uint64_t dropped = invert_block_regs(d, kb, limit);
   if (threadIdx.x == 0 && dropped) atomicAdd(ndrop, __popcll(dropped));
   store_pivot(d, kb, dropped, P);
 }
@@ -235,39 +277,6 @@ __device__ __forceinline__ void mma_m16n8k8_tf32(float (&d)[4], const uint32_t (
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
-template <class T>
-struct V4 {
-  T v[4];
-};
-// four consecutive T (16-byte aligned; 32 for double)
-template <class T>
-__device__ __forceinline__ V4<T> ld4s(const T* p) {
-  V4<T> r;
-  if (sizeof(T) == 4) {
-    const float4 a = *reinterpret_cast<const float4*>(p);
-    r.v[0] = a.x;
-    r.v[1] = a.y;
-    r.v[2] = a.z;
-    r.v[3] = a.w;
-  } else {
-    const double2 a = *reinterpret_cast<const double2*>(p), b = *(reinterpret_cast<const double2*>(p) + 1);
-    r.v[0] = a.x;
-    r.v[1] = a.y;
-    r.v[2] = b.x;
-    r.v[3] = b.y;
-  }
-  return r;
-}
-template <class T>
-__device__ __forceinline__ void st4(T* p, const T (&v)[4]) {
-  if (sizeof(T) == 4) {
-    *reinterpret_cast<float4*>(p) = make_float4((float)v[0], (float)v[1], (float)v[2], (float)v[3]);
-  } else {
-    *reinterpret_cast<double2*>(p) = make_double2(v[0], v[1]);
-    *(reinterpret_cast<double2*>(p) + 1) = make_double2(v[2], v[3]);
-  }
-}
-
 // One sweep (pivot sub-tile kp = k0 / 64 of a 64-grid with n64 sub-tiles per
 // side): every sub-tile (a, b), a <= b, of the upper tiles, 64 x 64 per block,
 // 4 x 4 per thread:
@@ -302,6 +311,9 @@ __global__ void __launch_bounds__(256) k_sweep(T* __restrict__ tiles, int nt, in
   const int64_t i0 = (int64_t)a * NB, j0 = (int64_t)b * NB;
   const int ty = threadIdx.x >> 4, tx = threadIdx.x & 15;
   T* zt = tiles + tile_index(a >> 1, b >> 1, nt) * CT * CT + (a & 1) * NB * CT + (b & 1) * NB;
+  // the next pivot block's limits, ahead of their use (diag0 is padded to whole blocks)
+  T limit = (T)0;
+  if (has_next && blockIdx.x == 0 && threadIdx.x < NB) limit = pivot_limit<T>(tol * diag0[k0 + NB + threadIdx.x]);
   // R and Tm slices -> shared memory (16-byte chunks; rows of length ldr, a multiple of 64)
   constexpr int CH = NB * (int)sizeof(T) / 16;  // chunks per row
   for (int q = threadIdx.x; q < NB * CH; q += 256) {
@@ -418,9 +430,8 @@ __global__ void __launch_bounds__(256) k_sweep(T* __restrict__ tiles, int nt, in
     }
   }
   if (has_next && blockIdx.x == 0) {  // the next pivot block, already updated: invert it
-    __shared__ T rowp[2][NB], colp[2][NB];
     const int kbn = (int)((m0 - k0 - NB) < NB ? (m0 - k0 - NB) : NB);
-    const uint64_t dropped = invert_block_regs(d, kbn, rowp, colp, diag0 + k0 + NB, tol);
+    const uint64_t dropped = invert_block_regs(d, kbn, limit);
     if (threadIdx.x == 0 && dropped) atomicAdd(ndrop, __popcll(dropped));
     store_pivot(d, kbn, dropped, Pn);
   }
