@@ -1003,8 +1003,11 @@ __global__ void __launch_bounds__(NT) k_star_numeric(int S, char* pool, const in
 // pivots S holds -S^{-1}; S is SPD, so no pivoting) and rounded to the solve's precision
 // into the star's records.
 // Bound by the FP64 pipe (c^3 / 2 multiply-adds at two a cycle and SM), so the rank-1
-// updates from shared memory cost nothing extra.  A block of 256 threads takes a star; the
-// triangle lies in shared memory up to CORE_SMEM nodes, else in a slab of global memory.
+// updates from shared memory cost nothing extra; but a warp's FP64 instruction takes 16 cycles
+// however few of its lanes matter, so the division is left to the warps that hold the column and
+// the column is scaled once (every warp dividing and every row scaling its own factor cost more
+// than the updates of a 42-node block: 1.42 ms on the 3D workload, 0.85 now).  A block of 256
+// threads takes a star; the triangle lies in shared memory up to CORE_SMEM nodes, else in a slab of global memory.
 // ---------------------------------------------------------------------------
 constexpr int CORE_SMEM = 224;  // 224 * 225 / 2 * 8 B = 201,600 B
 // The rounded inverse S^{-1} + E, |E| <= eps |S^{-1}|, keeps its stiff modes only while eps k
@@ -1030,11 +1033,12 @@ __global__ void __launch_bounds__(256) k_star_core(int S, char* pool, const int6
     if (c <= lo || c > hi) continue;  // uniform over the block
     double* col = sm_core;            // the pivot's column
     double* dg = sm_core + c;         // S's diagonal
-    double* A = SMEM ? sm_core + 2 * c : slab + (int64_t)blockIdx.x * slab_n;  // row i at i (i + 1) / 2
+    double* uc = sm_core + 2 * c;     // -1 / pivot times the pivot's column
+    double* A = SMEM ? sm_core + 3 * c : slab + (int64_t)blockIdx.x * slab_n;  // row i at i (i + 1) / 2
     const int core0 = B.n - c;
     const int64_t tri = (int64_t)c * (c + 1) / 2;
     for (int64_t e = tid; e < tri; e += 256) {
-      int i = (int)((sqrt(8.0 * (double)e + 1.0) - 1.0) * 0.5);
+      int i = (int)((sqrtf(8.0f * (float)e + 1.0f) - 1.0f) * 0.5f);  // a guess
       while ((int64_t)i * (i + 1) / 2 > e) --i;
       while ((int64_t)(i + 1) * (i + 2) / 2 <= e) ++i;
       const int j = (int)(e - (int64_t)i * (i + 1) / 2);
@@ -1062,23 +1066,27 @@ __global__ void __launch_bounds__(256) k_star_core(int S, char* pool, const int6
     for (int i = tid; i < c; i += 256) dg[i] = A[(int64_t)i * (i + 1) / 2 + i];
     bool bad = false;
     for (int k = 0; k < c; ++k) {
-      double piv = A[(int64_t)k * (k + 1) / 2 + k];
-      if (!(piv > 0.0)) {
-        bad = true;
-        piv = 1.0;
-      }
-      const double ip = 1.0 / piv;
-      for (int i = tid; i < c; i += 256) {
-        const int hi2 = i > k ? i : k, lo2 = i > k ? k : i;
-        col[i] = A[(int64_t)hi2 * (hi2 + 1) / 2 + lo2];
+      if (tid < c) {
+        double piv = A[(int64_t)k * (k + 1) / 2 + k];
+        if (!(piv > 0.0)) {
+          bad = true;
+          piv = 1.0;
+        }
+        const double ip = 1.0 / piv;
+        for (int i = tid; i < c; i += 256) {
+          const int hi2 = i > k ? i : k, lo2 = i > k ? k : i;
+          const double v = A[(int64_t)hi2 * (hi2 + 1) / 2 + lo2];
+          col[i] = v;
+          uc[i] = i == k ? -ip : -v * ip;
+        }
       }
       __syncthreads();
       for (int i = wid; i < c; i += 8) {
         double* row = A + (int64_t)i * (i + 1) / 2;
         if (i == k) {
-          for (int j = lane; j <= i; j += 32) row[j] = j == k ? -ip : col[j] * ip;
+          for (int j = lane; j <= i; j += 32) row[j] = j == k ? uc[j] : -uc[j];
         } else {
-          const double u = -col[i] * ip;
+          const double u = uc[i];
           for (int j = lane; j <= i; j += 32) row[j] = j == k ? -u : fma(u, col[j], row[j]);
         }
       }
@@ -1121,7 +1129,7 @@ static int core_inverses_t(spnet_pc_s* pc, DevArena& tmp, int32_t* noinv, int* n
     return SPNET_OK;
   };
   if (csm > 0)
-    SPNET_TRY(launch(k_star_core<T, true>, pc->S, sizeof(double) * ((size_t)csm * (csm + 1) / 2 + 2 * csm), nullptr, 0, 0,
+    SPNET_TRY(launch(k_star_core<T, true>, pc->S, sizeof(double) * ((size_t)csm * (csm + 1) / 2 + 3 * csm), nullptr, 0, 0,
                      CORE_SMEM));
   if (nbig > 0) {
     const int64_t n = (int64_t)cmax * (cmax + 1) / 2;
@@ -1130,7 +1138,7 @@ static int core_inverses_t(spnet_pc_s* pc, DevArena& tmp, int32_t* noinv, int* n
     while (grid > 1 && grid * n * 8 > ((int64_t)2 << 30)) grid /= 2;
     double* slab = nullptr;
     SPNET_TRY(tmp.get(&slab, grid * n));
-    SPNET_TRY(launch(k_star_core<T, false>, grid, sizeof(double) * 2 * cmax, slab, n, CORE_SMEM, CORE_INV));
+    SPNET_TRY(launch(k_star_core<T, false>, grid, sizeof(double) * 3 * cmax, slab, n, CORE_SMEM, CORE_INV));
   }
   return SPNET_OK;
 }
