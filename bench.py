@@ -999,7 +999,7 @@ def main():
                                               "sums), times added (the star solve overlaps the others)")}
         roof["bytes_rule"] = ("algorithmic bytes per the per-iteration count of the method: index list, "
                               "r and results per star entry (20 B) and 2 v B per factor entry for the star "
-                              "solve; storage-format bytes (window descriptors, columns, headers, padding, "
+                              "solve; storage-format bytes (step and group headers, columns, padding, "
                               "tile padding, int64 row pointers) listed apart as format overhead")
     cpu = None
     if rank == 0 and not args.no_cpu_baseline:

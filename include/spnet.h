@@ -330,7 +330,7 @@ int spnet_server_poll(spnet_server_t server, int64_t ticket, spnet_result* resul
  * end (*cancelled = 0).  Errors: BAD_INPUT (unknown ticket). */
 int spnet_server_cancel(spnet_server_t server, int64_t ticket, int* cancelled);
 /* spnet_server_estimate -- the peak device bytes admission charges for a request (the
- * operator and its copies of K, star factors and solve windows, the dense A_0 and its
+ * operator and its copies of K, star factors and solve records, the dense A_0 and its
  * inverse, the PCG vectors and blocks).  Host only. */
 int spnet_server_estimate(const spnet_request* request, int64_t* bytes);
 /* spnet_server_budget -- the device bytes the server's running requests may hold. */

@@ -61,7 +61,7 @@ namespace spnet {
 
 // device bytes a request is estimated to need at its peak (set-up): the
 // operator and its copies of K, the preconditioner (star factors and solve
-// windows, corner tables, the dense A_0 and its inverse tiles), PCG vectors
+// records, corner tables, the dense A_0 and its inverse tiles), PCG vectors
 int64_t request_estimate(const spnet_request* r) {
   const int ndof = r->model == SPNET_MODEL_TRUSS3 ? 3 : 1;
   const int64_t n_dof = r->n_nodes * ndof;
