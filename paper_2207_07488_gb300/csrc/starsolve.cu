@@ -728,6 +728,7 @@ __global__ void __launch_bounds__(256, JW == 1 ? 6 : 4) k_star_solve(SolveArgs A
     oa = H->off[SLOTS];
     ob = H->off[SLOTS + 1];
   }
+  __syncwarp();  // warp 0 polls the mbarriers that its first lane has initialised
   int eo[8], es[8];
 #pragma unroll
   for (int e = 0; e < 8; ++e) {
