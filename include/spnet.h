@@ -258,6 +258,12 @@ int setup_preconditioner(spnet_op_t op, double H, const int* gamma_faces,
 int pcg_solve(spnet_op_t op, spnet_pc_t pc, int nrhs, const double* f, const double* g,
               double* x, int use_x0, double rtol, int maxit, int mem, spnet_stats* stats);
 
+/* spnet_op_wait_limit -- how long a star solve of the operator's preconditioners waits for a
+ * copy of its factor data, in SM clocks, from the next call on (at first 4e9, about 2 s).  A
+ * call whose wait runs out returns SPNET_ERR_TIMEOUT; with 0 every wait gives up at once, so
+ * that a caller can exercise that status.  Errors: BAD_INPUT (null operator, clocks < 0). */
+int spnet_op_wait_limit(spnet_op_t op, int64_t clocks);
+
 int spnet_op_destroy(spnet_op_t op);
 int spnet_pc_destroy(spnet_pc_t pc);
 

@@ -194,6 +194,12 @@ int pcg_solve(spnet_op_t op, spnet_pc_t pc, int nrhs, const double* f, const dou
   return spnet::pcg_run(op, pc, nrhs, f, g, x, use_x0, rtol, maxit, mem, stats);
 }
 
+int spnet_op_wait_limit(spnet_op_t op, int64_t clocks) {
+  if (!op || clocks < 0) return fail(SPNET_ERR_BAD_INPUT, "spnet_op_wait_limit: null operator or clocks < 0");
+  op->wait_clocks = clocks;
+  return SPNET_OK;
+}
+
 int spnet_op_destroy(spnet_op_t op) {
   cudaGetLastError();  // start from a clean error state
   if (!op) return SPNET_OK;

@@ -588,9 +588,12 @@ static void iteration(spnet_pc_s* pc, cudaStream_t s, cudaStream_t side, int par
 constexpr int CHUNK = 8;  // even: a chunk leaves the residual in pc->r
 static_assert(CHUNK % 2 == 0, "the residual buffers alternate per iteration");
 
-// the chunk of iterations as a CUDA graph (captured once per preconditioner)
+// the chunk of iterations as a CUDA graph (captured once per preconditioner and wait limit)
 static int chunk_graph(spnet_pc_s* pc, cudaStream_t s) {
-  if (pc->graph_exec) return SPNET_OK;
+  if (pc->graph_exec && pc->graph_wait == pc->op->wait_clocks) return SPNET_OK;
+  if (pc->graph_exec) cudaGraphExecDestroy(pc->graph_exec);  // captured with another wait limit
+  pc->graph_exec = nullptr;
+  pc->graph_wait = pc->op->wait_clocks;
   if (!pc->side) {
     SPNET_CUDA_TRY(cudaStreamCreateWithFlags(&pc->side, cudaStreamNonBlocking));
     SPNET_CUDA_TRY(cudaEventCreateWithFlags(&pc->ev_fork, cudaEventDisableTiming));

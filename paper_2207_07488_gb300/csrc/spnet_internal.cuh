@@ -98,6 +98,7 @@ enum : int { TUNE_STAR_MAP = 0, TUNE_SPMV_LANES = 1, TUNE_BATCH_JW = 2, TUNE_KIN
 struct TuneClass {
   int c[4];
 };
+constexpr int64_t WAIT_CLOCKS = 4000000000ll;  // limit of the kernels' waits: about 2 s
 // 1 and *value: the class's choice is known; 0: the caller measures it and reports it with
 // tune_end (value 0: failed).  Waits while another set-up measures the class.
 int tune_begin(int kind, const TuneClass& c, int* value);
@@ -129,6 +130,7 @@ struct spnet_op_s {
   int* dflags = nullptr;
   double* spmv_tmp = nullptr;   // [2*n_free] scratch for spnet_spmv on host arrays
   int refcount = 0;
+  int64_t wait_clocks = spnet::WAIT_CLOCKS;  // spnet_op_wait_limit
 };
 
 struct spnet_pc_s {
@@ -217,6 +219,7 @@ struct spnet_pc_s {
   int64_t* estar = nullptr;        // [n_elem*nc] base of the element's entries in w (-1: no star)
   spnet::Scal* scal = nullptr;
   cudaGraphExec_t graph_exec = nullptr;  // a chunk of PCG iterations
+  int64_t graph_wait = 0;                // the wait limit it was captured with
   cudaStream_t side = nullptr;     // second stream of the graph (star solves)
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
   int graph_launches = 0;

@@ -522,8 +522,9 @@ __device__ __forceinline__ void bulk_load(unsigned dst, const void* src, unsigne
                "l"(src), "r"(bytes), "r"(bar)
                : "memory");
 }
-// true once the phase of the given parity is complete; gives up after 4e9 clocks (2 s)
-__device__ __forceinline__ bool mbar_wait(unsigned bar, unsigned parity) {
+// true once the phase of the given parity is complete; gives up after `limit` clocks (0: at once)
+__device__ __forceinline__ bool mbar_wait(unsigned bar, unsigned parity, long long limit) {
+  if (limit <= 0) return false;
   long long t0 = 0;
   for (int it = 0;; ++it) {
     unsigned ok;
@@ -534,7 +535,7 @@ __device__ __forceinline__ bool mbar_wait(unsigned bar, unsigned parity) {
         : "memory");
     if (ok) return true;
     if (it == 0) t0 = clock64();
-    else if (clock64() - t0 > 4000000000ll) return false;
+    else if (clock64() - t0 > limit) return false;
   }
 }
 
@@ -683,6 +684,7 @@ struct SolveArgs {
   const uint16_t* iperm;
   int rec_size, ylen;
   int wr;                  // warps of a team
+  long long wait;          // clocks a wait for a record may take (spnet_op_wait_limit)
   int* err;                // set where a wait ran out
 };
 
@@ -739,7 +741,7 @@ __global__ void __launch_bounds__(256, JW == 1 ? 6 : 4) k_star_solve(SolveArgs A
   pdl_trigger();
   if (done && *done) {
     if (tid == 0)  // the copies in flight end before the block does
-      for (int i = 0; i < SLOTS && i < nrec; ++i) mbar_wait(bars + 8 * i, 0u);
+      for (int i = 0; i < SLOTS && i < nrec; ++i) mbar_wait(bars + 8 * i, 0u, WAIT_CLOCKS);
     return;
   }
   const double alpha = q ? sc->alpha : 0.0;
@@ -779,12 +781,12 @@ __global__ void __launch_bounds__(256, JW == 1 ? 6 : 4) k_star_solve(SolveArgs A
   for (int rec = 0; rec < nrec; ++rec) {
     // one warp polls, the barrier tells the rest; it is also the barrier after the previous
     // record's last step (or the gather)
-    const bool ok = tid >= 32 || mbar_wait(bars + 8 * sl, phase);
+    const bool ok = tid >= 32 || mbar_wait(bars + 8 * sl, phase, A.wait);
     if (__syncthreads_or(!ok)) {
       if (tid == 0) {
         *A.err = 1;
         for (int u = 0; u < SLOTS && rec + u < nrec; ++u)  // every copy in flight (phases as issued)
-          mbar_wait(bars + 8 * ((sl + u) % SLOTS), sl + u < SLOTS ? phase : phase ^ 1u);
+          mbar_wait(bars + 8 * ((sl + u) % SLOTS), sl + u < SLOTS ? phase : phase ^ 1u, WAIT_CLOCKS);
       }
       return;
     }
@@ -897,7 +899,8 @@ static int launch_solve_t(spnet_pc_s* pc, int wr, int teams, const double* r, co
     attr_set[dev] = true;
   }
   const int groups = (k + JW * teams - 1) / (JW * teams);
-  SolveArgs A{(const StarHdr*)pc->shdr, pc->srec, pc->rec_off, pc->iperm_star, pc->rec_size, pc->ylen, wr, err};
+  SolveArgs A{(const StarHdr*)pc->shdr, pc->srec, pc->rec_off, pc->iperm_star, pc->rec_size, pc->ylen, wr,
+              pc->op->wait_clocks, err};
   launch_pdl(k_star_solve<T, JW>, (unsigned)(pc->S * groups), wr * teams * 32, (size_t)solve_smem(pc, JW, teams), s, A,
              r, q, sc, done, k, groups, w);
   return SPNET_OK;

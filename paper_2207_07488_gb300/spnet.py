@@ -41,7 +41,7 @@ EXPORTED = [
     "spnet_server_create", "spnet_server_submit", "spnet_server_wait", "spnet_server_destroy",
     "spnet_pc_apply_batch", "spnet_server_poll", "spnet_server_cancel", "spnet_server_estimate",
     "spnet_server_budget", "spnet_tune_cache_load", "spnet_tune_cache_save", "spnet_tune_cache_clear",
-    "spnet_tune_counts", "spnet_assemble_beam",
+    "spnet_tune_counts", "spnet_assemble_beam", "spnet_op_wait_limit",
 ]
 KERNELS = ["spmv", "update", "restrict", "stars", "coarse", "combine", "direction",
            "star_symbolic", "star_numeric", "sweep", "galerkin"]
@@ -121,6 +121,7 @@ def load(build_if_missing: bool = True):
     lib.setup_preconditioner.argtypes = [P, dbl, C.POINTER(C.c_int), C.POINTER(Options), C.POINTER(P)]
     lib.pcg_solve.argtypes = [P, P, i32, P, P, P, i32, dbl, i32, i32, C.POINTER(Stats)]
     lib.spnet_op_destroy.argtypes = [P]
+    lib.spnet_op_wait_limit.argtypes = [P, i64]
     lib.spnet_pc_destroy.argtypes = [P]
     lib.spnet_last_error.argtypes = [C.c_char_p, C.c_size_t]
     lib.spnet_op_get_info.argtypes = [P, C.POINTER(OpInfo)]
@@ -354,6 +355,10 @@ class Operator:
         y = np.zeros(self.info.n_free)
         _check(self._lib.spnet_spmv(self.handle, xp, y.ctypes.data, mem))
         return y
+
+    def wait_limit(self, clocks=4_000_000_000):
+        """spnet_op_wait_limit: SM clocks a star solve waits for its data before ERR_TIMEOUT."""
+        _check(self._lib.spnet_op_wait_limit(self.handle, int(clocks)))
 
     def close(self):
         if self.handle:
