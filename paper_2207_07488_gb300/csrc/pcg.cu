@@ -706,6 +706,7 @@ int export_item(spnet_pc_s* pc, int what, void* host_buf) {
 
 int pc_apply_free(spnet_pc_s* pc, const double* r_free, double* z_free, int which) {
   cudaStream_t s = pc->op->stream;
+  SPNET_CUDA_TRY(cudaMemsetAsync(&pc->scal->err, 0, sizeof(int), s));  // an earlier call's
   to_pc(pc, r_free, pc->vtmp);
   if (which == 0) precond_any(pc, pc->vtmp, pc->z, 1, 1, 0, s);
   else if (which == 1) precond_any(pc, pc->vtmp, pc->z, 1, 0, 0, s);

@@ -47,6 +47,19 @@ def test_every_call_with_star_solves_reports_a_wait_that_ran_out(handles):
         np.testing.assert_array_equal(c(), b)
 
 
+@pytest.mark.parametrize("failing", ["solve", "apply", "stars"])
+def test_an_apply_after_a_timeout_reports_its_own_waits_only(handles, failing):
+    p, op, pc = handles
+    r = np.random.default_rng(2).standard_normal(op.info.n_free)
+    z, w = pc.apply(r), pc.stars(r)
+    op.wait_limit(0)
+    _timeout({"solve": lambda: spnet.pcg_solve(op, pc, p.f, p.dirichlet_vals),
+              "apply": lambda: pc.apply(r), "stars": lambda: pc.stars(r)}[failing])
+    op.wait_limit()
+    np.testing.assert_array_equal(pc.apply(r), z)
+    np.testing.assert_array_equal(pc.stars(r), w)
+
+
 def test_a_negative_limit_is_refused(handles):
     _, op, _ = handles
     with pytest.raises(spnet.SpnetError) as e:
