@@ -1008,6 +1008,17 @@ int star_records_fill(spnet_pc_s* pc) {
   return SPNET_OK;
 }
 
+// SPNET_ERR_TIMEOUT where a wait of the solves just timed ran out: their times say nothing.  The
+// flag is cleared, so that it is not charged to the first call on the preconditioner.
+static int timed_waits(spnet_pc_s* pc) {
+  cudaStream_t s = pc->op->stream;
+  int err = 0;
+  SPNET_CUDA_TRY(cudaMemcpyAsync(&err, &pc->scal->err, sizeof(int), cudaMemcpyDeviceToHost, s));
+  SPNET_CUDA_TRY(cudaMemsetAsync(&pc->scal->err, 0, sizeof(int), s));
+  SPNET_CUDA_TRY(cudaStreamSynchronize(s));
+  return err ? fail(SPNET_ERR_TIMEOUT, "setup_preconditioner: a device wait of the timed star solves ran out") : SPNET_OK;
+}
+
 int star_map_tune(spnet_pc_s* pc) {
   if (pc->S == 0 || pc->star_map > 0) return SPNET_OK;  // fixed
   if (pc->S < 4 * num_sms()) return SPNET_OK;           // a few stars per SM: see star_records_fill
@@ -1047,6 +1058,7 @@ int star_map_tune(spnet_pc_s* pc) {
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
+  if (rc == SPNET_OK) rc = timed_waits(pc);
   pc->solve_wpb = best;
   tune_end(TUNE_STAR_MAP, key, rc == SPNET_OK ? best : 0);
   return rc;
@@ -1111,6 +1123,7 @@ int batch_jw_tune(spnet_pc_s* pc) {
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
+  if (rc == SPNET_OK) rc = timed_waits(pc);
   tune_end(TUNE_BATCH_JW, key, rc == SPNET_OK ? best : 0);
   pc->batch_jw = rc == SPNET_OK ? best : 0;
   return rc;

@@ -60,6 +60,24 @@ def test_an_apply_after_a_timeout_reports_its_own_waits_only(handles, failing):
     np.testing.assert_array_equal(pc.stars(r), w)
 
 
+@pytest.mark.parametrize("opts", [dict(), dict(star_map=4, batch_rhs=4)], ids=["warps", "columns"])
+def test_a_setup_whose_timed_solves_ran_out_fails_and_keeps_no_choice(opts):
+    # enough stars (four an SM) for the choice of warps to be timed
+    p = nw.scalar_band_problem(nw.fiber_network_2d(1000, 0.1, seed=7), 1.0 / 40)
+    op = spnet.Operator.from_problem(p)
+    spnet.tune_cache_clear()
+    op.wait_limit(0)
+    _timeout(lambda: spnet.Preconditioner(op, p.H, p.gamma_faces, **opts))
+    assert spnet.tune_counts() == (0, 0)
+    op.wait_limit()
+    pc = spnet.Preconditioner(op, p.H, p.gamma_faces, **opts)
+    assert pc.info.n_stars >= 4 * torch.cuda.get_device_properties(0).multi_processor_count
+    assert spnet.tune_counts() == (1, 0)
+    assert np.isfinite(pc.apply(np.ones(op.info.n_free))).all()
+    pc.close()
+    op.close()
+
+
 def test_a_negative_limit_is_refused(handles):
     _, op, _ = handles
     with pytest.raises(spnet.SpnetError) as e:
