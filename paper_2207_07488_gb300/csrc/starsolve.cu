@@ -31,6 +31,7 @@
 #include <atomic>
 
 #include "star_blob.cuh"
+#include "star_ring.cuh"
 
 namespace spnet {
 
@@ -38,7 +39,6 @@ constexpr int STEP_GROUPS = 16;
 constexpr int WIDE_K = 192;       // a row with more entries goes across the lanes
 constexpr int SOLVE_SMEM = 227 * 1024;
 constexpr int SOLVE_HEAD = 128;   // the slots' mbarriers
-constexpr int SLOTS = 3;
 
 // Record size.  A block waits and synchronises once a record, so a record holds eight columns of
 // the largest dense block where 16 KB allow it (a 16-byte column group, c * 16 bytes, always
@@ -785,8 +785,8 @@ __global__ void __launch_bounds__(256, JW == 1 ? 6 : 4) k_star_solve(SolveArgs A
     if (__syncthreads_or(!ok)) {
       if (tid == 0) {
         *A.err = 1;
-        for (int u = 0; u < SLOTS && rec + u < nrec; ++u)  // every copy in flight (phases as issued)
-          mbar_wait(bars + 8 * ((sl + u) % SLOTS), sl + u < SLOTS ? phase : phase ^ 1u, WAIT_CLOCKS);
+        for (int i = rec; i < ring_issued(rec, nrec); ++i)  // every copy in flight
+          mbar_wait(bars + 8 * (i % SLOTS), ring_parity(i), WAIT_CLOCKS);
       }
       return;
     }
