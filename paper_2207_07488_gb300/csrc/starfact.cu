@@ -83,6 +83,20 @@ __host__ __device__ inline uint32_t node_rank(uint32_t t) {
 
 __host__ __device__ inline int64_t core_entries(int core_max) { return (int64_t)core_max * (core_max - 1) / 2; }
 
+// The state of a star: its structure is to be built; built, the values are to come; done.
+enum : int32_t { STAR_DONE = 0, STAR_TODO = 1, STAR_BUILT = 2 };
+
+// What a pass over the stars counts.  Stars that did not fit their scratch or the pool, or whose
+// dense block is too ill conditioned to be inverted, are left for another pass.
+struct StarCount {
+  int next;       // the queue of stars
+  int left;       // stars left for another pass
+  int need_core;  // the largest dense block among them
+  int pad;
+  unsigned long long pool_top;   // bytes of the pool given out
+  unsigned long long pool_more;  // bytes the stars left will take
+};
+
 struct StarArgs {
   Mesh m;
   int S;
@@ -101,13 +115,13 @@ struct StarArgs {
   int core_max;    // largest dense block the scratch holds
   char* pool;
   int64_t pool_cap;
-  unsigned long long* pool_top;
   int64_t* star_off;
   int32_t* star_lev;
   int32_t* star_nnz;
   int32_t* star_core;
   int* flags;
-  int* next;
+  StarCount* cnt;
+  int32_t* todo;   // [S] STAR_*
   int core_inv;    // largest dense block that is inverted (0: none)
   const int32_t* noinv;  // [S] 1: a star whose block is not inverted (ill conditioned)
   int cap;            // adjacency slots per node (adjacency_cap)
@@ -162,6 +176,16 @@ __device__ inline Scratch carve(char* cold, char* hot, int nmax, int core_max, i
   return s;
 }
 
+// a star left for another pass: c nodes of its dense block as columns, of `nnz` entries the rest
+// (or all: block_in)
+__device__ inline void leave_star(const StarArgs& A, int flag, int n, int nlev, int nnz, int c, bool block_in = false) {
+  atomicOr(A.flags, flag);
+  atomicAdd(&A.cnt->left, 1);
+  atomicMax(&A.cnt->need_core, c);
+  atomicAdd(&A.cnt->pool_more,
+            (unsigned long long)blob_layout(n, nlev, nnz + (block_in ? 0 : (int)core_entries(c))).total);
+}
+
 __device__ inline int local_of_pc(const Mesh& m, const StarElems& se, const int32_t* elem_ptr,
                                   const int32_t* elem_of, int k_multi0, int k_multi1, int k_multi2,
                                   int j) {
@@ -211,9 +235,10 @@ __global__ void __launch_bounds__(128) k_star_symbolic(StarArgs A) {
   const unsigned FULL = 0xffffffffu;
   for (;;) {
     int s = 0;
-    if (lane == 0) s = atomicAdd(A.next, 1);
+    if (lane == 0) s = atomicAdd(&A.cnt->next, 1);
     s = __shfl_sync(FULL, s, 0);
     if (s >= A.S) break;
+    if (A.todo[s] != STAR_TODO) continue;
     const int k = A.star_mesh[s];
     const int n = A.star_n[s];
     if (n > A.nmax || n > 65535) {
@@ -426,7 +451,7 @@ __global__ void __launch_bounds__(128) k_star_symbolic(StarArgs A) {
       core_c = c;
       inv = c <= core_inv;
       if (!inv && (c > A.core_max || ncol + core_entries(c) > (int64_t)A.nmax * CAP + core_entries(A.core_max))) {
-        if (lane == 0) atomicOr(A.flags, FLAG_STAR_BIG);
+        if (lane == 0) leave_star(A, FLAG_STAR_BIG, n, nlev + c, ncol, c);
         continue;
       }
       if (inv) {
@@ -469,10 +494,10 @@ __global__ void __launch_bounds__(128) k_star_symbolic(StarArgs A) {
     // place the blob
     const BlobLayout L = blob_layout(n, nlev, ncol);
     unsigned long long off = 0;
-    if (lane == 0) off = atomicAdd(A.pool_top, (unsigned long long)L.total);
+    if (lane == 0) off = atomicAdd(&A.cnt->pool_top, (unsigned long long)L.total);
     off = __shfl_sync(FULL, off, 0);
     if ((int64_t)off + L.total > A.pool_cap) {
-      if (lane == 0) atomicOr(A.flags, FLAG_POOL);
+      if (lane == 0) leave_star(A, FLAG_POOL, n, nlev, ncol, inv ? 0 : core_c, true);
       continue;
     }
     char* blob = A.pool + off;
@@ -486,6 +511,7 @@ __global__ void __launch_bounds__(128) k_star_symbolic(StarArgs A) {
       A.star_lev[s] = nlev + (inv ? 1 : 0);
       A.star_nnz[s] = ncol;
       A.star_core[s] = core_c;
+      A.todo[s] = STAR_BUILT;
     }
     int32_t* gidx = (int32_t*)(blob + L.gidx);
     uint16_t* perm = (uint16_t*)(blob + L.perm);
@@ -583,10 +609,12 @@ __global__ void __launch_bounds__(BT) k_star_symbolic_block(StarArgs A) {
     __syncthreads();
   };
   for (;;) {
-    if (tid == 0) sh_i[0] = atomicAdd(A.next, 1);
+    __syncthreads();  // the previous star's last reads of sh_i
+    if (tid == 0) sh_i[0] = atomicAdd(&A.cnt->next, 1);
     __syncthreads();
     const int s = sh_i[0];
     if (s >= A.S) break;
+    if (A.todo[s] != STAR_TODO) continue;
     const int k = A.star_mesh[s];
     const int n = A.star_n[s];
     const StarElems se = star_elems(A.m, k, A.elem_ptr);
@@ -781,8 +809,7 @@ __global__ void __launch_bounds__(BT) k_star_symbolic_block(StarArgs A) {
       core_c = c;
       inv = c <= core_inv;
       if (!inv && (c > A.core_max || ncol + core_entries(c) > (int64_t)A.nmax * CAP + core_entries(A.core_max))) {
-        if (tid == 0) atomicOr(A.flags, FLAG_STAR_BIG);
-        __syncthreads();
+        if (tid == 0) leave_star(A, FLAG_STAR_BIG, n, nlev + c, ncol, c);
         continue;
       }
       place_rest(false);
@@ -825,12 +852,11 @@ __global__ void __launch_bounds__(BT) k_star_symbolic_block(StarArgs A) {
     for (int t = tid; t < n; t += BT) W.rcnt[t] = 0;
     // place the blob
     const BlobLayout L = blob_layout(n, nlev, ncol);
-    if (tid == 0) sh_off = atomicAdd(A.pool_top, (unsigned long long)L.total);
+    if (tid == 0) sh_off = atomicAdd(&A.cnt->pool_top, (unsigned long long)L.total);
     __syncthreads();
     const unsigned long long off = sh_off;
     if ((int64_t)off + L.total > A.pool_cap) {
-      if (tid == 0) atomicOr(A.flags, FLAG_POOL);
-      __syncthreads();
+      if (tid == 0) leave_star(A, FLAG_POOL, n, nlev, ncol, inv ? 0 : core_c, true);
       continue;
     }
     char* blob = A.pool + off;
@@ -844,6 +870,7 @@ __global__ void __launch_bounds__(BT) k_star_symbolic_block(StarArgs A) {
       A.star_lev[s] = nlev + (inv ? 1 : 0);
       A.star_nnz[s] = ncol;
       A.star_core[s] = core_c;
+      A.todo[s] = STAR_BUILT;
     }
     int32_t* gidx = (int32_t*)(blob + L.gidx);
     uint16_t* perm = (uint16_t*)(blob + L.perm);
@@ -921,12 +948,13 @@ __device__ __forceinline__ void group_sync() {
 }
 
 template <int TPS>
-__global__ void __launch_bounds__(NT) k_star_numeric(int S, char* pool, const int64_t* star_off,
+__global__ void __launch_bounds__(NT) k_star_numeric(int S, char* pool, const int64_t* star_off, const int32_t* todo,
                                                      const int64_t* kptr, const int32_t* kcol,
                                                      const double* kval, int* flags) {
   constexpr int GPB = NT / TPS;  // stars per block at a time
   const int tid = threadIdx.x % TPS;
   for (int64_t s = (int64_t)blockIdx.x * GPB + threadIdx.x / TPS; s < S; s += (int64_t)gridDim.x * GPB) {
+    if (todo[s] != STAR_BUILT) continue;  // uniform over the group
     const Blob B = blob_at(pool + star_off[s]);
     const int nlev = B.nlev;
     const int32_t *gidx = B.gidx, *c2r = B.c2r;
@@ -1024,7 +1052,7 @@ __global__ void __launch_bounds__(256) k_star_core(int S, char* pool, const int6
                                                    const double* __restrict__ kval, const int64_t* __restrict__ coff,
                                                    const int32_t* __restrict__ ckc, char* __restrict__ recs,
                                                    double* slab, int64_t slab_n, int lo, int hi, int32_t* noinv,
-                                                   int* n_ill, int* flags) {
+                                                   int32_t* todo, StarCount* cnt, int* flags) {
   extern __shared__ __align__(16) double sm_core[];
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   for (int s = blockIdx.x; s < S; s += gridDim.x) {
@@ -1098,7 +1126,11 @@ __global__ void __launch_bounds__(256) k_star_core(int S, char* pool, const int6
       ill |= !(dg[i] * -A[(int64_t)i * (i + 1) / 2 + i] <= (sizeof(T) == 4 ? KAPPA32 : KAPPA64));
     if (__syncthreads_or(ill) && tid == 0) {
       noinv[s] = 1;
-      atomicAdd(n_ill, 1);
+      todo[s] = STAR_TODO;
+      atomicAdd(&cnt->left, 1);
+      atomicMax(&cnt->need_core, c);
+      // (fewer where the elimination had stopped for the block: it goes on without one)
+      atomicAdd(&cnt->pool_more, (unsigned long long)blob_layout(B.n, B.nlev + c, B.nnz + (int)core_entries(c)).total);
     }
     T* out = (T*)(recs + coff[s]);
     const int kc = ckc[s], cp = (c + 3) / 4 * 4;
@@ -1112,7 +1144,7 @@ __global__ void __launch_bounds__(256) k_star_core(int S, char* pool, const int6
 }
 
 template <class T>
-static int core_inverses_t(spnet_pc_s* pc, DevArena& tmp, int32_t* noinv, int* n_ill, int* flags) {
+static int core_inverses_t(spnet_pc_s* pc, DevArena& tmp, int32_t* noinv, int32_t* todo, StarCount* cnt) {
   cudaStream_t s = pc->op->stream;
   int cmax = 0, csm = 0, nbig = 0;  // largest block; largest that fits shared memory; blocks beyond
   for (int c : pc->star_inv) {
@@ -1124,7 +1156,7 @@ static int core_inverses_t(spnet_pc_s* pc, DevArena& tmp, int32_t* noinv, int* n
     SPNET_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
     note_launch();
     kern<<<grid, 256, smem, s>>>(pc->S, pc->pool, pc->star_off, pc->K.ptr, pc->K.col, pc->K.val, pc->core_off,
-                                 pc->core_kc, pc->srec, slab, slab_n, lo, hi, noinv, n_ill, flags);
+                                 pc->core_kc, pc->srec, slab, slab_n, lo, hi, noinv, todo, cnt, pc->op->dflags);
     SPNET_CUDA_TRY(cudaGetLastError());
     return SPNET_OK;
   };
@@ -1143,38 +1175,51 @@ static int core_inverses_t(spnet_pc_s* pc, DevArena& tmp, int32_t* noinv, int* n
   return SPNET_OK;
 }
 
-static int core_inverses(spnet_pc_s* pc, DevArena& tmp, int32_t* noinv, int* n_ill, int* flags) {
-  return pc->precision == SPNET_PREC_FP64 ? core_inverses_t<double>(pc, tmp, noinv, n_ill, flags)
-                                          : core_inverses_t<float>(pc, tmp, noinv, n_ill, flags);
+static int core_inverses(spnet_pc_s* pc, DevArena& tmp, int32_t* noinv, int32_t* todo, StarCount* cnt) {
+  return pc->precision == SPNET_PREC_FP64 ? core_inverses_t<double>(pc, tmp, noinv, todo, cnt)
+                                          : core_inverses_t<float>(pc, tmp, noinv, todo, cnt);
 }
 
-// *ill: stars whose dense block is too ill conditioned to be inverted, marked in noinv (the
-// caller comes again with the marks)
-static int factor_stars(spnet_pc_s* pc, int32_t* noinv, int* ill) {
+// what the passes of the factorisation share
+struct StarWork {
+  int acap = 0;                // adjacency slots per node
+  int core_max = 0;            // largest dense block the scratch takes as columns
+  int left = 0;                // stars whose structure is to be built
+  int32_t* noinv = nullptr;    // [S] 1: the dense block is not inverted
+  int32_t* todo = nullptr;     // [S] STAR_*
+  StarCount* cnt = nullptr;
+};
+
+// room for `more` bytes behind the first `used` (a multiple of 16, as blobs and the pool are) of
+// the pool, which are kept
+static int pool_room(spnet_pc_s* pc, const StarWork& W, int64_t used, int64_t more) {
   cudaStream_t s = pc->op->stream;
-  if (pc->sum_s > INT32_MAX)
-    return fail(SPNET_ERR_UNSUPPORTED, "setup_preconditioner: the stars hold more than 2^31-1 entries in total");
-  if (pc->max_star > 65535)  // u16 places
-    return fail(SPNET_ERR_UNSUPPORTED, "setup_preconditioner: a star holds more than 65535 dofs");
+  more = align_up(more, 16);
+  if (used + more > pc->pool_bytes) {
+    char* p = nullptr;
+    SPNET_TRY(pc->mem.get(&p, used + more));
+    if (used > 0) SPNET_CUDA_TRY(cudaMemcpyAsync(p, pc->pool, used, cudaMemcpyDeviceToDevice, s));
+    if (pc->pool) pc->mem.release(pc->pool);
+    pc->pool = p;
+    pc->pool_bytes = used + more;
+  }
+  const unsigned long long top = (unsigned long long)used;
+  SPNET_CUDA_TRY(cudaMemcpyAsync(&W.cnt->pool_top, &top, sizeof(top), cudaMemcpyHostToDevice, s));
+  SPNET_CUDA_TRY(cudaStreamSynchronize(s));  // top goes out of scope
+  return SPNET_OK;
+}
+
+// the structures of the stars to do.  Stars that do not fit the scratch or the pool are
+// counted, and the pass repeated for them alone with what they need.
+static int star_structures(spnet_pc_s* pc, StarWork& W) {
+  cudaStream_t s = pc->op->stream;
   DevArena tmp;
   tmp.stream = s;
   struct Guard {
     DevArena& a;
     ~Guard() { a.free_all(); }
   } guard{tmp};
-  const int nmax = pc->max_star;
-  int max_row = 0;
-  {
-    int* d = nullptr;
-    SPNET_TRY(tmp.get(&d, 1));
-    SPNET_CUDA_TRY(cudaMemsetAsync(d, 0, sizeof(int), s));
-    note_launch();
-    k_max_row<<<4 * num_sms(), 256, 0, s>>>(pc->N, pc->K.ptr, d);
-    SPNET_CUDA_TRY(cudaGetLastError());
-    SPNET_CUDA_TRY(cudaMemcpyAsync(&max_row, d, sizeof(int), cudaMemcpyDeviceToHost, s));
-    SPNET_CUDA_TRY(cudaStreamSynchronize(s));
-  }
-  const int acap = adjacency_cap(max_row - 1, pc->d, pc->max_star);
+  const int nmax = pc->max_star, acap = W.acap;
   const int64_t hot = hot_bytes(nmax, acap);
   // a warp per star with everything in shared memory when four warps' worth fit in 200 KiB,
   // else a block of four warps per star (its marks in shared memory while they fit)
@@ -1196,45 +1241,23 @@ static int factor_stars(spnet_pc_s* pc, int32_t* noinv, int* ill) {
       attr_set[dev] = true;
     }
   }
-  // per-warp scratch, with room for the columns of a dense block of core_max nodes where it
-  // is not inverted; warps within a 1 GiB budget.  (Without inverses, stars beyond 4 CORE_FIRST
-  // dofs start at four times the capacity: a failed first pass costs a launch.)
-  const int vb = pc->precision == SPNET_PREC_FP64 ? 8 : 4;
-  const int core_inv = !pc->panels ? 0 : (int64_t)pc->max_star * vb > STAR_HUGE ? 256 : CORE_INV;
-  pc->core_inv = core_inv;
-  int core_max = core_inv > 0 ? 0
-                 : nmax <= 4 * CORE_FIRST ? (nmax < CORE_FIRST ? nmax : CORE_FIRST)
-                                          : 4 * CORE_FIRST;
-  int64_t stride = 0, workers = 0;  // scratch of a worker (a warp or a block)
+  int* flags = pc->op->dflags;
   char* scratch = nullptr;
-  auto size_scratch = [&]() -> int {
-    stride = cold_bytes(nmax, core_max, acap) + (per_warp ? 0 : align_up(hot, 256));
-    workers = (int64_t)(per_warp ? 4 : 1) * per_sm * num_sms();
+  for (int attempt = 0; attempt < 8; ++attempt) {
+    // per-worker scratch (a warp or a block), with room for the columns of a dense block of
+    // core_max nodes where it is not inverted; workers within a 1 GiB budget
+    const int64_t stride = cold_bytes(nmax, W.core_max, acap) + (per_warp ? 0 : align_up(hot, 256));
+    int64_t workers = (int64_t)(per_warp ? 4 : 1) * per_sm * num_sms();
     const int64_t budget = (int64_t)1 << 30;
     if (workers * stride > budget) workers = budget / stride;
-    if (workers > pc->S) workers = pc->S;
+    if (workers > W.left) workers = W.left;
     if (workers < 1) workers = 1;
     if (per_warp) workers = (workers + 3) / 4 * 4;
     if (scratch) tmp.release(scratch);
     scratch = nullptr;
-    return tmp.get(&scratch, workers * stride);
-  };
-  SPNET_TRY(size_scratch());
-  int* counters = nullptr;  // [0] next star, [2..3] pool top (u64)
-  SPNET_TRY(tmp.get(&counters, 4));
-  SPNET_TRY(pc->mem.get(&pc->star_off, pc->S));
-  SPNET_TRY(pc->mem.get(&pc->star_lev, pc->S));
-  SPNET_TRY(pc->mem.get(&pc->star_nnz, pc->S));
-  SPNET_TRY(pc->mem.get(&pc->star_core, pc->S));
-  // pool estimate: per dof 28 bytes + ~4 factor entries of 32 bytes, per star 64
-  int64_t cap = pc->sum_s * (28 + 4 * 32) + (int64_t)pc->S * 64 + (1 << 20);
-  int* flags = pc->op->dflags;
-  for (int attempt = 0; attempt < 8; ++attempt) {
-    if (pc->pool) pc->mem.release(pc->pool);
-    pc->pool = nullptr;
-    SPNET_TRY(pc->mem.get(&pc->pool, cap));
-    pc->pool_bytes = cap;
-    SPNET_CUDA_TRY(cudaMemsetAsync(counters, 0, sizeof(int) * 4, s));
+    SPNET_TRY(tmp.get(&scratch, workers * stride));
+    SPNET_CUDA_TRY(cudaMemsetAsync(W.cnt, 0, offsetof(StarCount, pool_top), s));
+    SPNET_CUDA_TRY(cudaMemsetAsync(&W.cnt->pool_more, 0, sizeof(unsigned long long), s));
     SPNET_CUDA_TRY(cudaMemsetAsync(flags, 0, sizeof(int), s));
     StarArgs A;
     A.m = mesh_of_pc(pc);
@@ -1251,110 +1274,152 @@ static int factor_stars(spnet_pc_s* pc, int32_t* noinv, int* ill) {
     A.hot = hot;
     A.hot_in_smem = hot_in_smem;
     A.nmax = nmax;
-    A.core_max = core_max;
+    A.core_max = W.core_max;
     A.pool = pc->pool;
-    A.pool_cap = cap;
-    A.pool_top = (unsigned long long*)(counters + 2);
+    A.pool_cap = pc->pool_bytes;
     A.star_off = pc->star_off;
     A.star_lev = pc->star_lev;
     A.star_nnz = pc->star_nnz;
     A.star_core = pc->star_core;
     A.flags = flags;
-    A.next = counters;
-    A.core_inv = core_inv;
-    A.noinv = noinv;
+    A.cnt = W.cnt;
+    A.todo = W.todo;
+    A.core_inv = pc->core_inv;
+    A.noinv = W.noinv;
     A.cap = acap;
     A.patch = pc->star_rule;
     A.q1w = pc->patch_w;
     A.N = pc->N;
     note_launch();
-    ProfScope ps(KID_STAR_SYMBOLIC, s);
-    if (per_warp) k_star_symbolic<<<(unsigned)(workers / 4), 128, smem, s>>>(A);
-    else k_star_symbolic_block<<<(unsigned)workers, BT, smem, s>>>(A);
+    {
+      ProfScope ps(KID_STAR_SYMBOLIC, s);
+      if (per_warp) k_star_symbolic<<<(unsigned)(workers / 4), 128, smem, s>>>(A);
+      else k_star_symbolic_block<<<(unsigned)workers, BT, smem, s>>>(A);
+    }
     SPNET_CUDA_TRY(cudaGetLastError());
     int h = 0;
+    StarCount c;
     SPNET_CUDA_TRY(cudaMemcpyAsync(&h, flags, sizeof(int), cudaMemcpyDeviceToHost, s));
+    SPNET_CUDA_TRY(cudaMemcpyAsync(&c, W.cnt, sizeof(c), cudaMemcpyDeviceToHost, s));
     SPNET_CUDA_TRY(cudaStreamSynchronize(s));
-    if (h & FLAG_POOL) {
-      cap *= 3;
-      continue;
-    }
-    if ((h & FLAG_STAR_BIG) && !(h & ~(FLAG_STAR_BIG | FLAG_POOL)) && core_max < nmax) {
-      // a dense block beyond the scratch: again with four times the capacity
-      core_max = core_max > 0 ? 4 * core_max : 4 * CORE_INV;
-      if (core_max > nmax) core_max = nmax;
-      SPNET_TRY(size_scratch());
-      continue;
-    }
-    if (h) return check_flags(flags, s, "setup_preconditioner (star structure)");
-    break;
+    if (h == 0) return SPNET_OK;
+    if ((h & ~(FLAG_STAR_BIG | FLAG_POOL)) || c.left == 0) break;
+    W.left = c.left;
+    W.core_max = c.need_core > W.core_max ? c.need_core : W.core_max;
+    // blobs lie below the first one that did not fit
+    const int64_t used = h & FLAG_POOL ? pc->pool_bytes : (int64_t)c.pool_top;
+    SPNET_TRY(pool_room(pc, W, used, (int64_t)c.pool_more));
   }
-  {
-    int h = 0;
-    SPNET_CUDA_TRY(cudaMemcpyAsync(&h, flags, sizeof(int), cudaMemcpyDeviceToHost, s));
-    SPNET_CUDA_TRY(cudaStreamSynchronize(s));
-    if (h) return check_flags(flags, s, "setup_preconditioner (star pool)");
-  }
-  note_launch();
-  ProfScope ps(KID_STAR_NUMERIC, s);
-  // a warp per star, or a block per star when some star exceeds 1024 dofs
-  if (pc->max_star > 1024)
-    k_star_numeric<NT><<<pc->S, NT, 0, s>>>(pc->S, pc->pool, pc->star_off, pc->K.ptr, pc->K.col, pc->K.val, flags);
-  else
-    k_star_numeric<32><<<(pc->S + NT / 32 - 1) / (NT / 32), NT, 0, s>>>(pc->S, pc->pool, pc->star_off, pc->K.ptr,
-                                                                        pc->K.col, pc->K.val, flags);
-  SPNET_CUDA_TRY(cudaGetLastError());
-  // the records of the solves: their sizes and places, the inverses of the dense blocks
-  // (written into them), then the sparse entries; the set-up blobs are released
-  std::vector<int32_t> lev(pc->S), nz(pc->S);
-  SPNET_CUDA_TRY(cudaMemcpyAsync(lev.data(), pc->star_lev, sizeof(int32_t) * pc->S, cudaMemcpyDeviceToHost, s));
-  SPNET_CUDA_TRY(cudaMemcpyAsync(nz.data(), pc->star_nnz, sizeof(int32_t) * pc->S, cudaMemcpyDeviceToHost, s));
-  SPNET_CUDA_TRY(cudaStreamSynchronize(s));
-  SPNET_TRY(star_records_plan(pc, tmp, lev, nz, noinv));
-  SPNET_CUDA_TRY(cudaMemsetAsync(counters, 0, sizeof(int), s));
-  SPNET_TRY(core_inverses(pc, tmp, noinv, counters, flags));
-  SPNET_CUDA_TRY(cudaMemcpyAsync(ill, counters, sizeof(int), cudaMemcpyDeviceToHost, s));
-  SPNET_TRY(check_flags(flags, s, "setup_preconditioner (star factorisation)"));
-  if (*ill > 0) return SPNET_OK;
-  // statistics
-  pc->factor_nnz = 0;
-  pc->total_levels = 0;
-  pc->max_levels = 0;
-  pc->panel_stars = 0;
-  for (int i = 0; i < pc->S; ++i) {
-    pc->factor_nnz += nz[i] + (int64_t)pc->star_inv[i] * (pc->star_inv[i] - 1) / 2;
-    pc->total_levels += lev[i];
-    pc->max_levels = lev[i] > pc->max_levels ? lev[i] : pc->max_levels;
-    pc->panel_stars += pc->star_inv[i] >= CORE_TC && pc->batch_rhs >= 2 && pc->precision == SPNET_PREC_MIXED;
-  }
-  SPNET_TRY(star_records_fill(pc));
-  pc->mem.release(pc->pool);
-  pc->pool = nullptr;
-  return SPNET_OK;
+  return check_flags(flags, s, "setup_preconditioner (star structure)");
 }
 
+// Stars whose dense block turns out too ill conditioned to be inverted (k_star_core) are
+// marked and done again, they alone; the others keep their factors.  (The mixed beam set-ups of
+// Section 6.3 mark stars with blocks of up to 1024 nodes; the larger blocks, most of the numeric
+// pass, are not inverted in the first place.  Every star done twice, the pull at H = 1/16 took
+// 27.1 s in mixed precision, now 13.1; each pass over all stars until the scratch and the pool
+// held the largest, 13.8 s in FP64, now 11.3.)
 int pc_factor_stars(spnet_pc_s* pc) {
   if (pc->S == 0) return SPNET_OK;
   cudaStream_t s = pc->op->stream;
+  if (pc->sum_s > INT32_MAX)
+    return fail(SPNET_ERR_UNSUPPORTED, "setup_preconditioner: the stars hold more than 2^31-1 entries in total");
+  if (pc->max_star > 65535)  // u16 places
+    return fail(SPNET_ERR_UNSUPPORTED, "setup_preconditioner: a star holds more than 65535 dofs");
   DevArena tmp;
   tmp.stream = s;
   struct Guard {
     DevArena& a;
     ~Guard() { a.free_all(); }
   } guard{tmp};
-  int32_t* noinv = nullptr;
-  SPNET_TRY(tmp.get(&noinv, pc->S));
-  SPNET_CUDA_TRY(cudaMemsetAsync(noinv, 0, sizeof(int32_t) * pc->S, s));
+  StarWork W;
+  SPNET_TRY(tmp.get(&W.noinv, pc->S));
+  SPNET_TRY(tmp.get(&W.todo, pc->S));
+  SPNET_TRY(tmp.get(&W.cnt, 1));
+  SPNET_CUDA_TRY(cudaMemsetAsync(W.noinv, 0, sizeof(int32_t) * pc->S, s));
+  fill_i32(W.todo, pc->S, STAR_TODO, s);
+  W.left = pc->S;
+  int max_row = 0;
+  {
+    int* d = nullptr;
+    SPNET_TRY(tmp.get(&d, 1));
+    SPNET_CUDA_TRY(cudaMemsetAsync(d, 0, sizeof(int), s));
+    note_launch();
+    k_max_row<<<4 * num_sms(), 256, 0, s>>>(pc->N, pc->K.ptr, d);
+    SPNET_CUDA_TRY(cudaGetLastError());
+    SPNET_CUDA_TRY(cudaMemcpyAsync(&max_row, d, sizeof(int), cudaMemcpyDeviceToHost, s));
+    SPNET_CUDA_TRY(cudaStreamSynchronize(s));
+  }
+  W.acap = adjacency_cap(max_row - 1, pc->d, pc->max_star);
+  const int vb = pc->precision == SPNET_PREC_FP64 ? 8 : 4;
+  pc->core_inv = !pc->panels ? 0 : (int64_t)pc->max_star * vb > STAR_HUGE ? 256 : CORE_INV;
+  // without inverses room for a dense block from the start: a repeated pass costs a launch
+  if (pc->core_inv == 0) {
+    const int first = pc->max_star <= 4 * CORE_FIRST ? CORE_FIRST : 4 * CORE_FIRST;
+    W.core_max = pc->max_star < first ? pc->max_star : first;
+  }
+  SPNET_TRY(pc->mem.get(&pc->star_off, pc->S));
+  SPNET_TRY(pc->mem.get(&pc->star_lev, pc->S));
+  SPNET_TRY(pc->mem.get(&pc->star_nnz, pc->S));
+  SPNET_TRY(pc->mem.get(&pc->star_core, pc->S));
+  // pool estimate: per dof 28 bytes + ~4 factor entries of 32 bytes, per star 64
+  SPNET_TRY(pool_room(pc, W, 0, pc->sum_s * (28 + 4 * 32) + (int64_t)pc->S * 64 + (1 << 20)));
+  int* flags = pc->op->dflags;
+  std::vector<int32_t> lev(pc->S), nz(pc->S);
   for (;;) {
-    int ill = 0;
-    SPNET_TRY(factor_stars(pc, noinv, &ill));
-    if (ill == 0) return SPNET_OK;
-    // the marked stars keep their block in the triangular factors (marks are only added, so
-    // this ends; in practice after one more pass)
-    for (void* p : {(void*)pc->pool, (void*)pc->star_off, (void*)pc->star_lev, (void*)pc->star_nnz,
-                    (void*)pc->star_core, (void*)pc->srec, (void*)pc->rec_off})
-      pc->mem.release(p);
-    pc->pool = nullptr;
+    SPNET_TRY(star_structures(pc, W));
+    note_launch();
+    {
+      ProfScope ps(KID_STAR_NUMERIC, s);
+      // a warp per star, or a block per star when some star exceeds 1024 dofs
+      if (pc->max_star > 1024)
+        k_star_numeric<NT><<<pc->S, NT, 0, s>>>(pc->S, pc->pool, pc->star_off, W.todo, pc->K.ptr, pc->K.col, pc->K.val,
+                                                flags);
+      else
+        k_star_numeric<32><<<(pc->S + NT / 32 - 1) / (NT / 32), NT, 0, s>>>(pc->S, pc->pool, pc->star_off, W.todo,
+                                                                            pc->K.ptr, pc->K.col, pc->K.val, flags);
+    }
+    SPNET_CUDA_TRY(cudaGetLastError());
+    SPNET_CUDA_TRY(cudaMemsetAsync(W.todo, 0, sizeof(int32_t) * pc->S, s));  // STAR_DONE
+    // the records of the solves: their sizes and places, the inverses of the dense blocks
+    // (written into them), then the sparse entries; the set-up blobs are released
+    SPNET_CUDA_TRY(cudaMemcpyAsync(lev.data(), pc->star_lev, sizeof(int32_t) * pc->S, cudaMemcpyDeviceToHost, s));
+    SPNET_CUDA_TRY(cudaMemcpyAsync(nz.data(), pc->star_nnz, sizeof(int32_t) * pc->S, cudaMemcpyDeviceToHost, s));
+    SPNET_CUDA_TRY(cudaStreamSynchronize(s));
+    DevArena pass;
+    pass.stream = s;
+    Guard pass_guard{pass};
+    SPNET_TRY(star_records_plan(pc, pass, lev, nz, W.noinv));
+    StarCount c{};
+    SPNET_CUDA_TRY(cudaMemcpyAsync(&c, W.cnt, sizeof(c), cudaMemcpyDeviceToHost, s));
+    SPNET_CUDA_TRY(cudaStreamSynchronize(s));
+    const int64_t used = (int64_t)c.pool_top;
+    SPNET_CUDA_TRY(cudaMemsetAsync(W.cnt, 0, sizeof(StarCount), s));
+    SPNET_TRY(core_inverses(pc, pass, W.noinv, W.todo, W.cnt));
+    SPNET_CUDA_TRY(cudaMemcpyAsync(&c, W.cnt, sizeof(c), cudaMemcpyDeviceToHost, s));
+    SPNET_TRY(check_flags(flags, s, "setup_preconditioner (star factorisation)"));  // waits for the device
+    if (c.left == 0) {
+      // statistics
+      pc->factor_nnz = 0;
+      pc->total_levels = 0;
+      pc->max_levels = 0;
+      pc->panel_stars = 0;
+      for (int i = 0; i < pc->S; ++i) {
+        pc->factor_nnz += nz[i] + (int64_t)pc->star_inv[i] * (pc->star_inv[i] - 1) / 2;
+        pc->total_levels += lev[i];
+        pc->max_levels = lev[i] > pc->max_levels ? lev[i] : pc->max_levels;
+        pc->panel_stars += pc->star_inv[i] >= CORE_TC && pc->batch_rhs >= 2 && pc->precision == SPNET_PREC_MIXED;
+      }
+      SPNET_TRY(star_records_fill(pc));
+      pc->mem.release(pc->pool);
+      pc->pool = nullptr;
+      return SPNET_OK;
+    }
+    W.left = c.left;
+    W.core_max = c.need_core > W.core_max ? c.need_core : W.core_max;
+    pc->mem.release(pc->srec);
+    pc->mem.release(pc->rec_off);
+    SPNET_TRY(pool_room(pc, W, used, (int64_t)c.pool_more));
   }
 }
 
