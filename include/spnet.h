@@ -337,7 +337,8 @@ int spnet_server_poll(spnet_server_t server, int64_t ticket, spnet_result* resul
 int spnet_server_cancel(spnet_server_t server, int64_t ticket, int* cancelled);
 /* spnet_server_estimate -- the peak device bytes admission charges for a request (the
  * operator and its copies of K, star factors and solve records, the dense A_0 and its
- * inverse, the PCG vectors and blocks).  Host only. */
+ * inverse, the PCG vectors and blocks).  Host only; reads coords and edges for the sizes of
+ * the stars (null: taken as evenly spread). */
 int spnet_server_estimate(const spnet_request* request, int64_t* bytes);
 /* spnet_server_budget -- the device bytes the server's running requests may hold. */
 int spnet_server_budget(spnet_server_t server, int64_t* bytes);

@@ -12,10 +12,12 @@
 // overlaps on the GPU (different streams).  Nothing a request computes depends
 // on what else runs: every kernel reduces in a fixed order, so a result is the
 // same alone and in the mix.
+#include <algorithm>
 #include <chrono>
 #include <condition_variable>
 #include <cstring>
 #include <deque>
+#include <exception>
 #include <map>
 #include <mutex>
 #include <thread>
@@ -59,6 +61,67 @@ struct spnet_server_s {
 
 namespace spnet {
 
+// The sizes (dofs) of a request's stars, from its nodes' elements; without coordinates, or with a
+// mesh no set-up takes, stars of the mean size.  Dirichlet dofs are counted too.
+static std::vector<int32_t> star_sizes(const spnet_request* r, int ndof) {
+  int n[3] = {1, 1, 1};
+  int64_t elems = 1;
+  const bool known = r->coords != nullptr;
+  for (int a = 0; a < r->dim; ++a) {
+    const double q = r->domain_hi[a] / r->H;
+    if (!(q >= 0.5 && q < 1e6)) return {};
+    n[a] = (int)(q + 0.5);
+    elems *= n[a];
+    if (elems > (1 << 22)) return {};
+  }
+  std::vector<int32_t> count(elems, 0);
+  if (known) {
+    for (int64_t i = 0; i < r->n_nodes; ++i) {
+      int64_t e = 0, stride = 1;
+      for (int a = 0; a < r->dim; ++a) {
+        const double s = r->coords[i * r->dim + a] * n[a] / r->domain_hi[a];
+        const int ea = s >= 0.0 ? (s < n[a] ? (int)s : n[a] - 1) : 0;  // (not a number: 0)
+        e += ea * stride;
+        stride *= n[a];
+      }
+      ++count[e];
+    }
+  } else {
+    std::fill(count.begin(), count.end(), (int32_t)((r->n_nodes + elems - 1) / elems));
+  }
+  const int lo = r->opts.star_set == SPNET_STARS_ALL ? 0 : 1;
+  std::vector<int32_t> sizes;
+  for (int k2 = r->dim == 3 ? lo : 0; k2 <= (r->dim == 3 ? n[2] - lo : 0); ++k2)
+    for (int k1 = lo; k1 <= n[1] - lo; ++k1)
+      for (int k0 = lo; k0 <= n[0] - lo; ++k0) {
+        const int k[3] = {k0, k1, k2};
+        int64_t dofs = 0;
+        for (int c = 0; c < 1 << r->dim; ++c) {
+          int64_t e = 0, stride = 1;
+          for (int a = 0; a < r->dim && e >= 0; ++a) {
+            const int ea = k[a] - 1 + (c >> a & 1);
+            e = ea < 0 || ea >= n[a] ? -1 : e + ea * stride;
+            stride *= n[a];
+          }
+          if (e >= 0) dofs += (int64_t)ndof * count[e];
+        }
+        if (dofs > 0) sizes.push_back((int32_t)std::min<int64_t>(dofs, 65535));  // more: refused by the set-up
+      }
+  return sizes;
+}
+
+// entries of the longest row of K
+static int longest_row(const spnet_request* r, int ndof) {
+  if (!r->edges) return 1;
+  std::vector<int32_t> deg(r->n_nodes, 0);
+  int32_t most = 0;
+  for (int64_t i = 0; i < 2 * r->n_edges; ++i) {
+    const int64_t v = r->edges[i];
+    if (v >= 0 && v < r->n_nodes) most = std::max(most, ++deg[v]);  // (others are refused later)
+  }
+  return ndof * (most + 1);
+}
+
 // device bytes a request is estimated to need at its peak (set-up): the
 // operator and its copies of K, the preconditioner (star factors and solve
 // records, corner tables, the dense A_0 and its inverse tiles), PCG vectors
@@ -69,12 +132,21 @@ int64_t request_estimate(const spnet_request* r) {
   int64_t m0 = ndof;
   for (int a = 0; a < r->dim; ++a) m0 *= (int64_t)(r->domain_hi[a] / r->H + 1.5);
   const int corners = 1 << r->dim;
-  int64_t b = 48 * nnz + n_dof * (256 + 96 * (int64_t)corners) + 20 * m0 * m0;
-  b += (int64_t)r->nrhs * n_dof * 24 + r->n_edges * 48 + (64ll << 20);
+  int64_t b = 48 * nnz + n_dof * (256 + 32 * (int64_t)corners) + 20 * m0 * m0;
+  if (r->dim == 2 || r->dim == 3) {
+    const double cycles = r->n_nodes > 0 ? std::max(0.0, (double)r->n_edges / r->n_nodes - 1.0) : 0.0;
+    try {
+      b += star_bytes_estimate(star_sizes(r, ndof), r->dim, ndof, longest_row(r, ndof), cycles,
+                               r->opts.precision == SPNET_PREC_FP64 ? 8 : 4, !r->opts.no_panels);
+    } catch (const std::exception&) {  // sizes beyond the host's memory: refused by the budget
+      b = INT64_MAX;
+    }
+  }
+  if (b < INT64_MAX) b += (int64_t)r->nrhs * n_dof * 24 + r->n_edges * 48 + (64ll << 20);
   // right-hand sides stepped together: five block vectors, the star results (about eight
   // entries per dof) and the coarse product's parts, for the block width
   const int64_t kb = r->nrhs < r->opts.batch_rhs ? r->nrhs : r->opts.batch_rhs;
-  if (kb >= 2) b += kb * n_dof * (40 + 64) + 2 * m0 * m0 + kb * 16 * m0;
+  if (kb >= 2 && b < INT64_MAX) b += kb * n_dof * (40 + 64) + 2 * m0 * m0 + kb * 16 * m0;
   return b;
 }
 

@@ -335,6 +335,8 @@ int pc_galerkin(spnet_pc_s* pc, double* A0_dense);
 
 // starfact.cu
 int pc_factor_stars(spnet_pc_s* pc);
+int64_t star_bytes_estimate(const std::vector<int32_t>& sizes, int dim, int ndof, int max_row, double cycles, int vb,
+                            int panels);
 // star solves for k <= 32 right-hand sides at once (R, W: [dofs][k]); W in the solve precision
 // (err: set where a wait ran out)
 int launch_star_batch(spnet_pc_s* pc, const double* R, int k, void* W, int* err, const int* done, cudaStream_t s);

@@ -1143,6 +1143,18 @@ __global__ void __launch_bounds__(256) k_star_core(int S, char* pool, const int6
   }
 }
 
+// Bytes of the structures' scratch, and of the slabs below, which come when it has been given back.
+constexpr int64_t SCRATCH_BUDGET = (int64_t)1 << 30;
+
+// Blocks of k_star_core with slabs of n doubles: two an SM (225 blocks of up to 623 nodes: set-up
+// 237 ms with two or four, 271 with one).
+static int slab_blocks(int64_t stars, int64_t n, int sms) {
+  int64_t g = 2ll * sms;
+  if (g > stars) g = stars;
+  if (g * n * 8 > SCRATCH_BUDGET) g = SCRATCH_BUDGET / (n * 8);
+  return g < 1 ? 1 : (int)g;
+}
+
 template <class T>
 static int core_inverses_t(spnet_pc_s* pc, DevArena& tmp, int32_t* noinv, int32_t* todo, StarCount* cnt) {
   cudaStream_t s = pc->op->stream;
@@ -1165,9 +1177,7 @@ static int core_inverses_t(spnet_pc_s* pc, DevArena& tmp, int32_t* noinv, int32_
                      CORE_SMEM));
   if (nbig > 0) {
     const int64_t n = (int64_t)cmax * (cmax + 1) / 2;
-    int grid = 4 * num_sms();
-    if (grid > nbig) grid = nbig;
-    while (grid > 1 && grid * n * 8 > ((int64_t)2 << 30)) grid /= 2;
+    const int grid = slab_blocks(nbig, n, num_sms());
     double* slab = nullptr;
     SPNET_TRY(tmp.get(&slab, grid * n));
     SPNET_TRY(launch(k_star_core<T, false>, grid, sizeof(double) * 3 * cmax, slab, n, CORE_SMEM, CORE_INV));
@@ -1178,6 +1188,80 @@ static int core_inverses_t(spnet_pc_s* pc, DevArena& tmp, int32_t* noinv, int32_
 static int core_inverses(spnet_pc_s* pc, DevArena& tmp, int32_t* noinv, int32_t* todo, StarCount* cnt) {
   return pc->precision == SPNET_PREC_FP64 ? core_inverses_t<double>(pc, tmp, noinv, todo, cnt)
                                           : core_inverses_t<float>(pc, tmp, noinv, todo, cnt);
+}
+
+// How the structures are spread over the GPU: a warp per star with everything in shared memory
+// when four warps' worth fit in 200 KiB, else a block of four warps per star (its marks in shared
+// memory while they fit).
+struct StructurePlan {
+  int nmax, acap, per_sm, hot_in_smem;
+  bool per_warp;
+  int64_t hot;
+  size_t smem;
+  StructurePlan(int nmax_, int acap_) : nmax(nmax_), acap(acap_), hot(hot_bytes(nmax_, acap_)) {
+    per_warp = 4 * hot <= 200 * 1024;
+    const int64_t marks = (BT / 32) * bitmap_bytes(nmax) + marks_bytes(nmax);
+    hot_in_smem = per_warp || marks <= 200 * 1024 ? 1 : 0;
+    smem = per_warp ? (size_t)(4 * hot) : (size_t)(hot_in_smem ? marks : (BT / 32) * bitmap_bytes(nmax));
+    per_sm = (int)((200 * 1024) / (smem + 1024));  // blocks per SM
+    per_sm = per_sm < 1 ? 1 : per_sm > (per_warp ? 4 : 8) ? (per_warp ? 4 : 8) : per_sm;
+  }
+  // scratch of a worker (a warp or a block), with room for the columns of a dense block of
+  // core_max nodes where it is not inverted
+  int64_t stride(int core_max) const {
+    return cold_bytes(nmax, core_max, acap) + (per_warp ? 0 : align_up(hot, 256));
+  }
+  int64_t workers(int core_max, int64_t stars, int sms) const {
+    int64_t w = (int64_t)(per_warp ? 4 : 1) * per_sm * sms;
+    if (w * stride(core_max) > SCRATCH_BUDGET) w = SCRATCH_BUDGET / stride(core_max);
+    if (w > stars) w = stars;
+    if (w < 1) w = 1;
+    return per_warp ? (w + 3) / 4 * 4 : w;
+  }
+};
+
+// the largest dense block that is inverted
+static int inverted_up_to(int panels, int max_star, int vb) {
+  return !panels ? 0 : (int64_t)max_star * vb > STAR_HUGE ? 256 : CORE_INV;
+}
+// the pool at first: per dof 28 bytes + ~4 factor entries of 32 bytes, per star 64
+static int64_t pool_first(int64_t dofs, int64_t stars) { return dofs * (28 + 4 * 32) + stars * 64 + (1 << 20); }
+
+// Device bytes that the stars' factors take at the peak of the set-up, estimated from the stars'
+// sizes; `cycles`: edges a node of the network beyond a tree's.  Not known before the elimination
+// are the factor entries (measured: 1.1 to 2 a dof on 3D networks, 4 to 8 in 2D and on trusses;
+// taken: 9) and the dense blocks (3D: up to n/6 with 0.1 cycles a node below 1000 dofs, where the
+// tail rule sets them, 0.05 n beyond; 0.22 n with 0.46; 2D: up to 7.4 sqrt n; taken: the tail
+// rule's or half of cycles * n in 3D, 8 sqrt n in 2D).
+int64_t star_bytes_estimate(const std::vector<int32_t>& sizes, int dim, int ndof, int max_row, double cycles, int vb,
+                            int panels) {
+  if (sizes.empty()) return 0;
+  const int64_t S = (int64_t)sizes.size();
+  int64_t sum = 0, nbig = 0, cbig = 0;
+  int nmax = 0;
+  for (int32_t n : sizes) {
+    sum += n;
+    nmax = n > nmax ? n : nmax;
+  }
+  const int core_inv = inverted_up_to(panels, nmax, vb);
+  double blocks = 0.0;
+  for (int32_t n : sizes) {
+    double c = dim == 2 ? 8.0 * std::sqrt((double)ndof * n) : 0.5 * cycles * n;
+    c = std::min(std::max(c, (double)tail_nodes(n)), (double)n);
+    // c^2 coefficients as an inverse, else entries of the records and the blob
+    blocks += c * c * (c <= core_inv ? vb : vb + 2 + 16);
+    if (c > CORE_SMEM && c <= core_inv) {
+      ++nbig;
+      cbig = std::max(cbig, (int64_t)c);
+    }
+  }
+  const StructurePlan P(nmax, adjacency_cap(max_row - 1, dim, nmax));
+  const int64_t scratch = P.workers(0, S, num_sms()) * P.stride(0);
+  const int64_t slab_n = cbig * (cbig + 1) / 2;
+  const int64_t slab = nbig > 0 ? slab_blocks(nbig, slab_n, num_sms()) * slab_n * 8 : 0;
+  const int64_t pool = pool_first(sum, S) + sum * (28 + 9 * 32);  // one that has grown, beside the old one
+  const int64_t records = sum * (2 * 10 * (vb + 2) + 6) + S * 512 + (int64_t)blocks;
+  return pool + std::max(scratch, records + slab);
 }
 
 // what the passes of the factorisation share
@@ -1203,9 +1287,20 @@ static int pool_room(spnet_pc_s* pc, const StarWork& W, int64_t used, int64_t mo
     pc->pool = p;
     pc->pool_bytes = used + more;
   }
+  if (used == 0) {
+    SPNET_CUDA_TRY(cudaMemsetAsync(&W.cnt->pool_top, 0, sizeof(W.cnt->pool_top), s));
+    return SPNET_OK;
+  }
   const unsigned long long top = (unsigned long long)used;
   SPNET_CUDA_TRY(cudaMemcpyAsync(&W.cnt->pool_top, &top, sizeof(top), cudaMemcpyHostToDevice, s));
   SPNET_CUDA_TRY(cudaStreamSynchronize(s));  // top goes out of scope
+  return SPNET_OK;
+}
+
+// nothing left, nothing asked for; the pool as it is
+static int clear_counts(const StarWork& W, cudaStream_t s) {
+  SPNET_CUDA_TRY(cudaMemsetAsync(W.cnt, 0, offsetof(StarCount, pool_top), s));
+  SPNET_CUDA_TRY(cudaMemsetAsync(&W.cnt->pool_more, 0, sizeof(W.cnt->pool_more), s));
   return SPNET_OK;
 }
 
@@ -1220,16 +1315,7 @@ static int star_structures(spnet_pc_s* pc, StarWork& W) {
     ~Guard() { a.free_all(); }
   } guard{tmp};
   const int nmax = pc->max_star, acap = W.acap;
-  const int64_t hot = hot_bytes(nmax, acap);
-  // a warp per star with everything in shared memory when four warps' worth fit in 200 KiB,
-  // else a block of four warps per star (its marks in shared memory while they fit)
-  const bool per_warp = 4 * hot <= 200 * 1024;
-  const int64_t marks = (BT / 32) * bitmap_bytes(nmax) + marks_bytes(nmax);
-  const int hot_in_smem = per_warp || marks <= 200 * 1024 ? 1 : 0;
-  const size_t smem = per_warp ? (size_t)(4 * hot)
-                               : (size_t)(hot_in_smem ? marks : (BT / 32) * bitmap_bytes(nmax));
-  int per_sm = (int)((200 * 1024) / (smem + 1024));  // blocks per SM
-  per_sm = per_sm < 1 ? 1 : per_sm > (per_warp ? 4 : 8) ? (per_warp ? 4 : 8) : per_sm;
+  const StructurePlan P(nmax, acap);
   {
     static std::atomic<bool> attr_set[64];  // per device
     int dev = 0;
@@ -1244,20 +1330,11 @@ static int star_structures(spnet_pc_s* pc, StarWork& W) {
   int* flags = pc->op->dflags;
   char* scratch = nullptr;
   for (int attempt = 0; attempt < 8; ++attempt) {
-    // per-worker scratch (a warp or a block), with room for the columns of a dense block of
-    // core_max nodes where it is not inverted; workers within a 1 GiB budget
-    const int64_t stride = cold_bytes(nmax, W.core_max, acap) + (per_warp ? 0 : align_up(hot, 256));
-    int64_t workers = (int64_t)(per_warp ? 4 : 1) * per_sm * num_sms();
-    const int64_t budget = (int64_t)1 << 30;
-    if (workers * stride > budget) workers = budget / stride;
-    if (workers > W.left) workers = W.left;
-    if (workers < 1) workers = 1;
-    if (per_warp) workers = (workers + 3) / 4 * 4;
+    const int64_t stride = P.stride(W.core_max), workers = P.workers(W.core_max, W.left, num_sms());
     if (scratch) tmp.release(scratch);
     scratch = nullptr;
     SPNET_TRY(tmp.get(&scratch, workers * stride));
-    SPNET_CUDA_TRY(cudaMemsetAsync(W.cnt, 0, offsetof(StarCount, pool_top), s));
-    SPNET_CUDA_TRY(cudaMemsetAsync(&W.cnt->pool_more, 0, sizeof(unsigned long long), s));
+    SPNET_TRY(clear_counts(W, s));
     SPNET_CUDA_TRY(cudaMemsetAsync(flags, 0, sizeof(int), s));
     StarArgs A;
     A.m = mesh_of_pc(pc);
@@ -1271,8 +1348,8 @@ static int star_structures(spnet_pc_s* pc, StarWork& W) {
     A.kval = pc->K.val;
     A.scratch = scratch;
     A.stride = stride;
-    A.hot = hot;
-    A.hot_in_smem = hot_in_smem;
+    A.hot = P.hot;
+    A.hot_in_smem = P.hot_in_smem;
     A.nmax = nmax;
     A.core_max = W.core_max;
     A.pool = pc->pool;
@@ -1293,8 +1370,8 @@ static int star_structures(spnet_pc_s* pc, StarWork& W) {
     note_launch();
     {
       ProfScope ps(KID_STAR_SYMBOLIC, s);
-      if (per_warp) k_star_symbolic<<<(unsigned)(workers / 4), 128, smem, s>>>(A);
-      else k_star_symbolic_block<<<(unsigned)workers, BT, smem, s>>>(A);
+      if (P.per_warp) k_star_symbolic<<<(unsigned)(workers / 4), 128, P.smem, s>>>(A);
+      else k_star_symbolic_block<<<(unsigned)workers, BT, P.smem, s>>>(A);
     }
     SPNET_CUDA_TRY(cudaGetLastError());
     int h = 0;
@@ -1352,7 +1429,7 @@ int pc_factor_stars(spnet_pc_s* pc) {
   }
   W.acap = adjacency_cap(max_row - 1, pc->d, pc->max_star);
   const int vb = pc->precision == SPNET_PREC_FP64 ? 8 : 4;
-  pc->core_inv = !pc->panels ? 0 : (int64_t)pc->max_star * vb > STAR_HUGE ? 256 : CORE_INV;
+  pc->core_inv = inverted_up_to(pc->panels, pc->max_star, vb);
   // without inverses room for a dense block from the start: a repeated pass costs a launch
   if (pc->core_inv == 0) {
     const int first = pc->max_star <= 4 * CORE_FIRST ? CORE_FIRST : 4 * CORE_FIRST;
@@ -1362,8 +1439,7 @@ int pc_factor_stars(spnet_pc_s* pc) {
   SPNET_TRY(pc->mem.get(&pc->star_lev, pc->S));
   SPNET_TRY(pc->mem.get(&pc->star_nnz, pc->S));
   SPNET_TRY(pc->mem.get(&pc->star_core, pc->S));
-  // pool estimate: per dof 28 bytes + ~4 factor entries of 32 bytes, per star 64
-  SPNET_TRY(pool_room(pc, W, 0, pc->sum_s * (28 + 4 * 32) + (int64_t)pc->S * 64 + (1 << 20)));
+  SPNET_TRY(pool_room(pc, W, 0, pool_first(pc->sum_s, pc->S)));
   int* flags = pc->op->dflags;
   std::vector<int32_t> lev(pc->S), nz(pc->S);
   for (;;) {
@@ -1391,10 +1467,7 @@ int pc_factor_stars(spnet_pc_s* pc) {
     Guard pass_guard{pass};
     SPNET_TRY(star_records_plan(pc, pass, lev, nz, W.noinv));
     StarCount c{};
-    SPNET_CUDA_TRY(cudaMemcpyAsync(&c, W.cnt, sizeof(c), cudaMemcpyDeviceToHost, s));
-    SPNET_CUDA_TRY(cudaStreamSynchronize(s));
-    const int64_t used = (int64_t)c.pool_top;
-    SPNET_CUDA_TRY(cudaMemsetAsync(W.cnt, 0, sizeof(StarCount), s));
+    SPNET_TRY(clear_counts(W, s));
     SPNET_TRY(core_inverses(pc, pass, W.noinv, W.todo, W.cnt));
     SPNET_CUDA_TRY(cudaMemcpyAsync(&c, W.cnt, sizeof(c), cudaMemcpyDeviceToHost, s));
     SPNET_TRY(check_flags(flags, s, "setup_preconditioner (star factorisation)"));  // waits for the device
@@ -1419,7 +1492,7 @@ int pc_factor_stars(spnet_pc_s* pc) {
     W.core_max = c.need_core > W.core_max ? c.need_core : W.core_max;
     pc->mem.release(pc->srec);
     pc->mem.release(pc->rec_off);
-    SPNET_TRY(pool_room(pc, W, used, (int64_t)c.pool_more));
+    SPNET_TRY(pool_room(pc, W, (int64_t)c.pool_top, (int64_t)c.pool_more));
   }
 }
 
