@@ -1052,7 +1052,7 @@ __global__ void __launch_bounds__(256) k_star_core(int S, char* pool, const int6
                                                    const double* __restrict__ kval, const int64_t* __restrict__ coff,
                                                    const int32_t* __restrict__ ckc, char* __restrict__ recs,
                                                    double* slab, int64_t slab_n, int lo, int hi, int32_t* noinv,
-                                                   int32_t* todo, StarCount* cnt, int* flags) {
+                                                   int32_t* todo, StarCount* cnt) {
   extern __shared__ __align__(16) double sm_core[];
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   for (int s = blockIdx.x; s < S; s += gridDim.x) {
@@ -1120,8 +1120,9 @@ __global__ void __launch_bounds__(256) k_star_core(int S, char* pool, const int6
       }
       __syncthreads();
     }
-    if (bad && tid == 0) atomicOr(flags, FLAG_NOT_SPD);
-    bool ill = false;
+    // a pivot lost to rounding (or a block that is not positive definite): the triangular factors
+    // decide
+    bool ill = bad;
     for (int i = tid; i < c; i += 256)
       ill |= !(dg[i] * -A[(int64_t)i * (i + 1) / 2 + i] <= (sizeof(T) == 4 ? KAPPA32 : KAPPA64));
     if (__syncthreads_or(ill) && tid == 0) {
@@ -1168,7 +1169,7 @@ static int core_inverses_t(spnet_pc_s* pc, DevArena& tmp, int32_t* noinv, int32_
     SPNET_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
     note_launch();
     kern<<<grid, 256, smem, s>>>(pc->S, pc->pool, pc->star_off, pc->K.ptr, pc->K.col, pc->K.val, pc->core_off,
-                                 pc->core_kc, pc->srec, slab, slab_n, lo, hi, noinv, todo, cnt, pc->op->dflags);
+                                 pc->core_kc, pc->srec, slab, slab_n, lo, hi, noinv, todo, cnt);
     SPNET_CUDA_TRY(cudaGetLastError());
     return SPNET_OK;
   };

@@ -74,3 +74,36 @@ def test_marked_stars_are_done_again_alone():
     flat.close()
     pc.close()
     op.close()
+
+
+def _nearly_singular(n, seed):
+    """A complete graph of n nodes in one star, tied to its Dirichlet node by less than the
+    rounding of its diagonal: whether the last pivot comes out positive is the rounding's choice."""
+    rng = np.random.default_rng(seed)
+    i, j = np.triu_indices(n, 1)
+    E = np.concatenate([np.stack([i, j], 1), [[0, n]]])
+    c = np.concatenate([rng.uniform(0.5, 2.0, len(i)), [1e-15]])
+    X = np.concatenate([rng.uniform(0.1, 0.9, (n, 2)), [[0.0, 0.5]]])
+    net = nw.Network(2, X, E.astype(np.int64), np.zeros(len(E), np.int8), c, c, np.zeros((len(E), 2)), (1.0, 1.0))
+    return nw.Problem(net, 1, "scalar", np.array([n], np.int64), np.zeros(1), np.ones(n + 1), 0.5, (0,))
+
+
+@pytest.mark.parametrize("prec", ["fp64", "mixed"])
+def test_a_pivot_lost_in_the_inverse_does_not_refuse_a_star_that_factors(prec):
+    pr = spnet.PREC_FP64 if prec == "fp64" else spnet.PREC_MIXED
+    taken = {True: 0, False: 0}
+    for seed in range(40):
+        p = _nearly_singular(40, seed)
+        op = spnet.Operator.from_problem(p)
+        ok = {}
+        for panels in (True, False):
+            try:
+                spnet.Preconditioner(op, 0.5, p.gamma_faces, precision=pr, panels=panels).close()
+                ok[panels] = True
+            except spnet.SpnetError as e:
+                assert e.code == spnet.ERR_NOT_SPD
+                ok[panels] = False
+        assert ok[True] or not ok[False], seed
+        taken[ok[False]] += 1
+        op.close()
+    assert taken[True] > 0 and taken[False] > 0  # both outcomes of the factorisation were met
