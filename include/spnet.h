@@ -353,7 +353,8 @@ int spnet_server_destroy(spnet_server_t server);
  * every set-up of a class uses the one measured value (a set-up meeting a class being
  * measured waits for it).  The cache can be saved and loaded, so that another process takes
  * the same choices without measuring: a text file of lines
- * "device<TAB>kind<TAB>c0,c1,c2,c3<TAB>value" (device: name, SM count, compute capability).
+ * "device<TAB>kind<TAB>c0,c1,c2,c3<TAB>value" (device: name, SM count, compute capability;
+ * kind: 1 lanes, 3 warps, 4 right-hand sides, others of earlier builds, kept but not read).
  * spnet_tune_cache_load  add the lines of a file to the cache.  Errors: BAD_INPUT (unreadable
  *                        file or malformed line; nothing is added then).
  * spnet_tune_cache_save  write the cache's measured entries (all devices) to a file.

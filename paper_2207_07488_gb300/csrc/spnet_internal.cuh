@@ -93,8 +93,10 @@ struct Scal {
 }  // namespace spnet
 struct spnet_pc_s;
 namespace spnet {
-// the tuner's cache (tune.cu): choices per device, kind and size class
-enum : int { TUNE_STAR_MAP = 0, TUNE_SPMV_LANES = 1, TUNE_BATCH_JW = 2, TUNE_KINDS = 3 };
+// the tuner's cache (tune.cu): choices per device, kind and size class.  Kinds 0 and 2 were the
+// choices of earlier star solves (stars a block, right-hand sides a warp): files that hold them
+// load, nothing reads them.
+enum : int { TUNE_SPMV_LANES = 1, TUNE_STAR_WARPS = 3, TUNE_STAR_COLUMNS = 4, TUNE_KINDS = 5 };
 struct TuneClass {
   int c[4];
 };

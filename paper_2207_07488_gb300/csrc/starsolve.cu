@@ -1004,7 +1004,7 @@ int star_records_fill(spnet_pc_s* pc) {
   int v = 0;
   if (pc->star_map > 0) pc->solve_wpb = pc->star_map;
   else if (S < 4 * num_sms()) pc->solve_wpb = 8;
-  else pc->solve_wpb = tune_peek(TUNE_STAR_MAP, map_class(pc), &v) ? known_warps(v) : 4;
+  else pc->solve_wpb = tune_peek(TUNE_STAR_WARPS, map_class(pc), &v) ? known_warps(v) : 4;
   return SPNET_OK;
 }
 
@@ -1025,7 +1025,7 @@ int star_map_tune(spnet_pc_s* pc) {
   const TuneClass key = map_class(pc);
   {
     int v = 0;
-    if (tune_begin(TUNE_STAR_MAP, key, &v)) {  // known
+    if (tune_begin(TUNE_STAR_WARPS, key, &v)) {  // known
       pc->solve_wpb = known_warps(v);
       return SPNET_OK;
     }
@@ -1035,7 +1035,7 @@ int star_map_tune(spnet_pc_s* pc) {
   if (cudaMemsetAsync(pc->vtmp, 0, sizeof(double) * pc->N, s) != cudaSuccess || cudaEventCreate(&e0) != cudaSuccess ||
       cudaEventCreate(&e1) != cudaSuccess) {
     if (e0) cudaEventDestroy(e0);
-    tune_end(TUNE_STAR_MAP, key, 0);
+    tune_end(TUNE_STAR_WARPS, key, 0);
     return fail(SPNET_ERR_CUDA, "setup_preconditioner: timing the star solve failed");
   }
   int best = 4, rc = SPNET_OK;
@@ -1060,7 +1060,7 @@ int star_map_tune(spnet_pc_s* pc) {
   cudaEventDestroy(e1);
   if (rc == SPNET_OK) rc = timed_waits(pc);
   pc->solve_wpb = best;
-  tune_end(TUNE_STAR_MAP, key, rc == SPNET_OK ? best : 0);
+  tune_end(TUNE_STAR_WARPS, key, rc == SPNET_OK ? best : 0);
   return rc;
 }
 
@@ -1076,7 +1076,7 @@ int batch_jw_tune(spnet_pc_s* pc) {
   const int vb = pc->precision == SPNET_PREC_FP64 ? 8 : 4;
   const TuneClass key{{vb * 64 + kp, half_octave(pc->S), half_octave(pc->max_star), pc->panel_stars > 0 ? 1 : 0}};
   int v = 0;
-  if (tune_begin(TUNE_BATCH_JW, key, &v)) {
+  if (tune_begin(TUNE_STAR_COLUMNS, key, &v)) {
     pc->batch_jw = v == 2 ? 2 : 4;  // whatever a loaded file holds
     return SPNET_OK;
   }
@@ -1090,7 +1090,7 @@ int batch_jw_tune(spnet_pc_s* pc) {
   const int64_t rbytes = 8ll * pc->N * k, wbytes = (int64_t)vb * pc->sum_s * k;
   int best = 4, rc = SPNET_OK;
   if (rbytes + wbytes > (2ll << 30)) {  // too large to time on the side: the default
-    tune_end(TUNE_BATCH_JW, key, best);
+    tune_end(TUNE_STAR_COLUMNS, key, best);
     pc->batch_jw = best;
     return SPNET_OK;
   }
@@ -1101,7 +1101,7 @@ int batch_jw_tune(spnet_pc_s* pc) {
       cudaMemsetAsync(R, 0, (size_t)rbytes, s) != cudaSuccess || cudaEventCreate(&e0) != cudaSuccess ||
       cudaEventCreate(&e1) != cudaSuccess) {
     if (e0) cudaEventDestroy(e0);
-    tune_end(TUNE_BATCH_JW, key, 0);
+    tune_end(TUNE_STAR_COLUMNS, key, 0);
     return rc ? rc : fail(SPNET_ERR_CUDA, "setup_preconditioner: timing the batched star solve failed");
   }
   float best_ms = 0.0f;
@@ -1124,7 +1124,7 @@ int batch_jw_tune(spnet_pc_s* pc) {
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   if (rc == SPNET_OK) rc = timed_waits(pc);
-  tune_end(TUNE_BATCH_JW, key, rc == SPNET_OK ? best : 0);
+  tune_end(TUNE_STAR_COLUMNS, key, rc == SPNET_OK ? best : 0);
   pc->batch_jw = rc == SPNET_OK ? best : 0;
   return rc;
 }

@@ -1,12 +1,12 @@
 // The tuner's cache: choices measured at set-up per device and size class.
 //
 // Three choices are timed on the preconditioner's own data the first time a
-// size class is met: the warps per block of the one-vector star solve, the
-// lanes per row of the SpMV, and the right-hand sides per warp of the batched
-// star solve.  The last two change the order of floating-point sums, so every
-// set-up of a class uses the one measured value: a set-up that meets a class
-// being measured waits for it, and a class is measured once per process (or
-// never, when a cache file saved earlier lists it).  The cache is kept per
+// size class is met: the warps that share a star of the one-vector star solve,
+// the lanes per row of the SpMV, and the right-hand sides per team of the
+// batched star solve.  The lanes change the order of floating-point sums, so
+// every set-up of a class uses the one measured value: a set-up that meets a
+// class being measured waits for it, and a class is measured once per process
+// (or never, when a cache file saved earlier lists it).  The cache is kept per
 // device (name, SM count, compute capability) and can be saved to and loaded
 // from a file of lines "device<TAB>kind<TAB>c0,c1,c2,c3<TAB>value".
 #include <condition_variable>
