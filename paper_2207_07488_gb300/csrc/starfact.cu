@@ -1144,15 +1144,15 @@ __global__ void __launch_bounds__(256) k_star_core(int S, char* pool, const int6
   }
 }
 
-// Bytes of the structures' scratch, and of the slabs below, which come when it has been given back.
-constexpr int64_t SCRATCH_BUDGET = (int64_t)1 << 30;
+// Bytes of the structures' scratch; and of the slabs below, which come when it has been given back.
+constexpr int64_t SCRATCH_BUDGET = (int64_t)1 << 30, SLAB_BUDGET = (int64_t)2 << 30;
 
-// Blocks of k_star_core with slabs of n doubles: two an SM (225 blocks of up to 623 nodes: set-up
-// 237 ms with two or four, 271 with one).
+// Blocks of k_star_core with slabs of n doubles: four an SM (29,791 blocks of 339 nodes on
+// average, 699 at most: set-up 5.9 s, 8.1 with two).
 static int slab_blocks(int64_t stars, int64_t n, int sms) {
-  int64_t g = 2ll * sms;
+  int64_t g = 4ll * sms;
   if (g > stars) g = stars;
-  if (g * n * 8 > SCRATCH_BUDGET) g = SCRATCH_BUDGET / (n * 8);
+  if (g * n * 8 > SLAB_BUDGET) g = SLAB_BUDGET / (n * 8);
   return g < 1 ? 1 : (int)g;
 }
 
@@ -1231,9 +1231,10 @@ static int64_t pool_first(int64_t dofs, int64_t stars) { return dofs * (28 + 4 *
 // Device bytes that the stars' factors take at the peak of the set-up, estimated from the stars'
 // sizes; `cycles`: edges a node of the network beyond a tree's.  Not known before the elimination
 // are the factor entries (measured: 1.1 to 2 a dof on 3D networks, 4 to 8 in 2D and on trusses;
-// taken: 9) and the dense blocks (3D: up to n/6 with 0.1 cycles a node below 1000 dofs, where the
-// tail rule sets them, 0.05 n beyond; 0.22 n with 0.46; 2D: up to 7.4 sqrt n; taken: the tail
-// rule's or half of cycles * n in 3D, 8 sqrt n in 2D).
+// taken: 9) and the dense blocks (3D: the tail rule's up to 1000 dofs, beyond up to 0.05 n with 0.1
+// cycles a node and 0.15 n with 0.46; 2D: up to 7.4 sqrt n; taken: the tail rule's or half of
+// cycles * n in 3D, 8 sqrt n in 2D).  Peak over estimate of whole requests: 0.06 to 0.75, 0.38 for
+// the 10.9M-node network.
 int64_t star_bytes_estimate(const std::vector<int32_t>& sizes, int dim, int ndof, int max_row, double cycles, int vb,
                             int panels) {
   if (sizes.empty()) return 0;
