@@ -103,8 +103,9 @@ typedef struct {
                         per block */
   int star_map;      /* warps that solve a star together in the one-vector star solve: 0 picks
                         it per size class (stars, largest star, bytes per star) by timing the
-                        candidates once per process (default); 1..8 fixes it.  A row is one
-                        lane's sum whatever the warps, so the choice changes no result */
+                        candidates once per process (eight, untimed, with fewer than four
+                        stars an SM; default); 1..8 fixes it.  A row is one lane's sum
+                        whatever the warps, so the choice changes no result */
   int patch;         /* SPNET_PATCH_* (default SPNET_PATCH_ELEMENT) */
   int no_panels;     /* 1: the dense block that ends a star's elimination is solved a node a
                         level; 0 (default): it is kept as its FP64 inverse, rounded to the

@@ -140,7 +140,7 @@ struct spnet_pc_s {
   spnet::DevArena mem;
   int precision = SPNET_PREC_MIXED, star_set = SPNET_STARS_INTERIOR, flexible = 1, max_restarts = 2;
   int batch_rhs = 1;            // right-hand sides pcg_solve steps together
-  int star_map = 0;             // warps per block of the star solve: 0 tuned per size class
+  int star_map = 0;             // warps that share a star of the one-vector solve: 0 tuned per size class
   int patch = SPNET_PATCH_ELEMENT;  // dofs a star holds (SPNET_PATCH_*)
   int coarse_space = SPNET_COARSE_Q1;  // SPNET_COARSE_*
   // The star kernels' patch test: a dof is off the star of the mesh node at its host element's

@@ -918,9 +918,11 @@ void launch_star_solve(spnet_pc_s* pc, const double* r, const double* q, const S
     launch_solve_t<float, 1>(pc, pc->solve_wpb, 1, r, q, sc, err, done, 1, (float*)pc->w, s);
 }
 
-// Widest block of right-hand sides stepped together.  It bounds the block vectors, so where
-// stars are large it stays at the width whose solve vectors, four (two, one) to a warp with
-// their places and 2 to 3 KB of factor data, fit a block's shared memory.
+// Widest block of right-hand sides stepped together, from what jw columns of the largest star took
+// in the solve's first layout (vectors, places and a few KB of factor data, in a block's shared
+// memory).  A block takes solve_smem now, and fewer columns where that does not fit; the widths and
+// the largest star (also in star_records_fill) are kept, so that the same stars are taken and the
+// same right-hand sides stepped together.
 static int64_t batch_bytes(const spnet_pc_s* pc, int jw) {
   const int64_t vb = pc->precision == SPNET_PREC_FP64 ? 8 : 4;
   return 8 * (80 + 32 * vb) + 80 + align_up(vb * pc->max_star * jw, 16) + align_up(2ll * pc->max_star, 16);
@@ -936,7 +938,7 @@ static int launch_batch_t(spnet_pc_s* pc, const double* R, int k, T* W, int* err
   int jw = pc->batch_jw > 0 ? pc->batch_jw : 4;
   if (k < jw) jw = k < 2 ? 1 : 2;
   while (jw > 1 && !solve_fits(pc, jw, 1)) jw /= 2;
-  // small stars: one warp a team, up to four teams on one ring; large ones: a team of four warps
+  // small stars: one warp a team, up to four teams on one ring; large ones: a team of eight warps
   const bool large = pc->max_star > 1024;
   const int wr = large ? 8 : 1;
   int teams = large ? 1 : 4;
@@ -997,7 +999,7 @@ int star_records_fill(spnet_pc_s* pc) {
   pc->rec_counts = nullptr;
   pc->rec_place = nullptr;
   pc->rec_first = pc->rec_base = nullptr;
-  // a vector of up to 200 KB less 2 to 3 KB
+  // a vector of up to 200 KB less a few (the limit of star_batch_max_k's layout)
   if (8 * (80 + 32 * vb) + 80 + align_up((int64_t)vb * pc->max_star, 16) > 200 * 1024 || !solve_fits(pc, 1, 1))
     return fail(SPNET_ERR_UNSUPPORTED, "setup_preconditioner: a star too large for the solve's shared memory");
   // a block per star: with few stars per SM eight warps shorten the longest star

@@ -20,7 +20,7 @@ def star_scale(o, r):
 def check_star_term(o, r, got, prec, sc=None):
     """Element-wise comparison of a star term with the oracle's.
 
-    FP64 (the same window kernels as FP32, on FP64 coefficients): every entry within
+    FP64 (the same kernels as FP32, on FP64 coefficients): every entry within
     1e-9 of the scale of the stars that hold it, so one wrong star anywhere fails by
     orders of magnitude.  Mixed (FP32 factors, condition numbers of the stars up to
     ~5e5): the relative error over every star's dofs within 1e-2, and over all

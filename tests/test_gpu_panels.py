@@ -1,9 +1,9 @@
-"""Dense blocks of large stars solved by panels on tensor cores (k right-hand sides, FP32).
+"""Dense blocks of large stars applied as their inverses (k right-hand sides, FP32).
 
 On a 2D network whose stars hold 1500-2000 dofs, the elimination of every star
-ends in a dense block of well over 32 nodes; with batch_rhs >= 2 the library
-solves those blocks by 16-row panels with tensor-core products instead of level
-by level.  Checked against the oracle (Section 4.1, eq. defPj: the exact local
+ends in a dense block of well over 32 nodes; the library applies those blocks as
+one product with their inverse instead of solving them a node a level.  Checked
+against the oracle (Section 4.1, eq. defPj: the exact local
 solves): the star term per column, per star within 1e-2 and over all dofs within
 2e-4 (the mixed-precision bounds of the other parity tests), whole batched
 solves to relative error 1e-6, agreement with the level-by-level solve of the
