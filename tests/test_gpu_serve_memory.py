@@ -17,12 +17,12 @@ if not torch.cuda.is_available():
 
 from paper_2207_07488_gb300 import spnet  # noqa: E402
 
-USED_HIGH = 8  # cudaMemPoolAttrUsedMemHigh
+USED_NOW, USED_HIGH = 7, 8  # cudaMemPoolAttrUsedMemCurrent, cudaMemPoolAttrUsedMemHigh
 
 
 @pytest.fixture(scope="module")
-def pool_high():
-    """pool_high(): the high-water mark of the default pool since the last call, which resets it."""
+def pool():
+    """pool(): (bytes of the default pool in use, their high-water mark since the last call)."""
     torch.zeros(1).cuda()
     for name in ("libcudart.so.13", "libcudart.so", "/usr/local/cuda/lib64/libcudart.so"):
         try:
@@ -32,14 +32,18 @@ def pool_high():
             rt = None
     if rt is None:
         pytest.skip("no CUDA runtime library to ask")
-    pool, v = C.c_void_p(), C.c_uint64(0)
-    assert rt.cudaDeviceGetDefaultMemPool(C.byref(pool), torch.cuda.current_device()) == 0
+    handle, v = C.c_void_p(), C.c_uint64(0)
+    assert rt.cudaDeviceGetDefaultMemPool(C.byref(handle), torch.cuda.current_device()) == 0
+
+    def get(attr):
+        assert rt.cudaMemPoolGetAttribute(handle, attr, C.byref(v)) == 0
+        return v.value
 
     def read():
-        assert rt.cudaMemPoolGetAttribute(pool, USED_HIGH, C.byref(v)) == 0
-        high, zero = v.value, C.c_uint64(0)
-        assert rt.cudaMemPoolSetAttribute(pool, USED_HIGH, C.byref(zero)) == 0
-        return high
+        torch.cuda.synchronize()
+        now, high, zero = get(USED_NOW), get(USED_HIGH), C.c_uint64(0)
+        assert rt.cudaMemPoolSetAttribute(handle, USED_HIGH, C.byref(zero)) == 0
+        return now, high
     return read
 
 
@@ -54,7 +58,7 @@ CASES = [("2d", 16, 224, 1, "mixed"), ("2d", 16, 224, 1, "fp64"), ("2d", 40, 0, 
 
 
 @pytest.mark.parametrize("kind,nH,block,k,prec", CASES)
-def test_the_peak_stays_below_the_estimate(pool_high, kind, nH, block, k, prec):
+def test_the_peak_stays_below_the_estimate(pool, kind, nH, block, k, prec):
     net = _net(kind)
     p = nw.truss_band_problem(net, 1.0 / nH) if kind == "truss" else nw.scalar_band_problem(net, 1.0 / nH)
     pr = spnet.PREC_FP64 if prec == "fp64" else spnet.PREC_MIXED
@@ -67,9 +71,9 @@ def test_the_peak_stays_below_the_estimate(pool_high, kind, nH, block, k, prec):
     F = np.random.default_rng(1).uniform(0.0, 1.0, (k, p.n_dof))
     est = spnet.request_estimate(p, f=F, precision=pr, batch_rhs=k)
     sv = spnet.Server(max_inflight=1)
-    pool_high()
+    held, _ = pool()  # by handles of other tests
     _, res = sv.wait(sv.submit(p, f=F, precision=pr, batch_rhs=k))
-    peak = pool_high()
+    peak = pool()[1] - held
     sv.close()
     assert res["status"] == spnet.OK, res["message"]
     assert 0 < peak <= est
