@@ -49,16 +49,20 @@ __host__ __device__ inline int switch_degree(int cap) { return cap - cap / 4; }
 // one product; larger ones (the beam model's largest stars) are eliminated a node a level.
 constexpr int CORE_INV = 1024;
 constexpr int CORE_FIRST = 256;  // capacity of the first attempt where blocks are not inverted
-                                 // (raised 4x on overflow)
 // Nodes left at which the elimination stops for the dense block.  Its inverse costs c^2
 // coefficients a solve and c^3 / 2 FP64 operations at set-up, and saves the levels of the last c
 // nodes, most of them of one or two rows.  One solve, 3D workload (341 dofs a star): 34 us with
 // 8 to 16 nodes, 33 with 24, 32 with 32, 34 with 48; structural workload (2,419 dofs): 168 us
 // with at most 64, 159 with 128, 170 with 192.
-__host__ __device__ inline int tail_nodes(int n) {
+// At most 128 (tail_most); 64 for 3D networks of few stars, where a star has its SM to itself and the
+// block's c^3 / 4 cycles are waited for, while the levels saved are few.  Set-up and one solve, 128 and
+// 64: 1,333 dofs in one star 2.68, 2.52 ms; 5,356 in 8 stars 3.77, 3.34, in 20 stars 3.73, 3.36;
+// 80,788 in 64 stars 21.2, 21.1; 110,699 in 125 stars 18.1, 18.5.  2D: 4,972 in 9 stars 6.35, 6.78.
+__host__ __device__ inline int tail_nodes(int n, int most) {
   const int t = n / 8;
-  return t < 32 ? 32 : t > 128 ? 128 : t;
+  return t < 32 ? 32 : t > most ? most : t;
 }
+inline int tail_most(int dim, int64_t stars, int sms) { return dim == 3 && 4 * stars <= sms ? 64 : 128; }
 
 // One elimination round takes an independent set among the nodes of degree at most
 // round_degree(md), md the least degree left.  A round is a level of the triangular
@@ -123,6 +127,7 @@ struct StarArgs {
   StarCount* cnt;
   int32_t* todo;   // [S] STAR_*
   int core_inv;    // largest dense block that is inverted (0: none)
+  int tail_most;   // see tail_nodes
   const int32_t* noinv;  // [S] 1: a star whose block is not inverted (ill conditioned)
   int cap;            // adjacency slots per node (adjacency_cap)
   int patch;          // SPNET_PATCH_*
@@ -272,7 +277,7 @@ __global__ void __launch_bounds__(128) k_star_symbolic(StarArgs A) {
     int npos = 0, nlev = 0, ncol = 0;
     bool dense = false;
     const int core_inv = A.noinv[s] ? 0 : A.core_inv;
-    const int tail = core_inv > 0 ? tail_nodes(n) : 0;
+    const int tail = core_inv > 0 ? tail_nodes(n, A.tail_most) : 0;
     while (npos < n) {
       if (n - npos <= tail) {
         dense = true;
@@ -643,7 +648,7 @@ __global__ void __launch_bounds__(BT) k_star_symbolic_block(StarArgs A) {
     int npos = 0, nlev = 0, ncol = 0;
     bool dense = false;
     const int core_inv = A.noinv[s] ? 0 : A.core_inv;
-    const int tail = core_inv > 0 ? tail_nodes(n) : 0;
+    const int tail = core_inv > 0 ? tail_nodes(n, A.tail_most) : 0;
     while (npos < n) {
       if (n - npos <= tail) {
         dense = true;
@@ -1249,7 +1254,7 @@ int64_t star_bytes_estimate(const std::vector<int32_t>& sizes, int dim, int ndof
   double blocks = 0.0;
   for (int32_t n : sizes) {
     double c = dim == 2 ? 8.0 * std::sqrt((double)ndof * n) : 0.5 * cycles * n;
-    c = std::min(std::max(c, (double)tail_nodes(n)), (double)n);
+    c = std::min(std::max(c, (double)tail_nodes(n, tail_most(dim, S, num_sms()))), (double)n);
     // c^2 coefficients as an inverse, else entries of the records and the blob
     blocks += c * c * (c <= core_inv ? vb : vb + 2 + 16);
     if (c > CORE_SMEM && c <= core_inv) {
@@ -1364,6 +1369,7 @@ static int star_structures(spnet_pc_s* pc, StarWork& W) {
     A.cnt = W.cnt;
     A.todo = W.todo;
     A.core_inv = pc->core_inv;
+    A.tail_most = tail_most(pc->d, pc->S, num_sms());
     A.noinv = W.noinv;
     A.cap = acap;
     A.patch = pc->star_rule;
