@@ -87,8 +87,9 @@ __host__ __device__ inline uint32_t node_rank(uint32_t t) {
 
 __host__ __device__ inline int64_t core_entries(int core_max) { return (int64_t)core_max * (core_max - 1) / 2; }
 
-// The state of a star: its structure is to be built; built, the values are to come; done.
-enum : int32_t { STAR_DONE = 0, STAR_TODO = 1, STAR_BUILT = 2 };
+// The state of a star: its structure is to be built; built, the values are to come; done (every
+// byte 1, as a memset sets it).
+enum : int32_t { STAR_TODO = 0, STAR_BUILT = 2, STAR_DONE = 0x01010101 };
 
 // What a pass over the stars counts.  Stars that did not fit their scratch or the pool, or whose
 // dense block is too ill conditioned to be inverted, are left for another pass.
@@ -96,9 +97,9 @@ struct StarCount {
   int next;       // the queue of stars
   int left;       // stars left for another pass
   int need_core;  // the largest dense block among them
-  int pad;
-  unsigned long long pool_top;   // bytes of the pool given out
+  int max_row;    // the longest row of K
   unsigned long long pool_more;  // bytes the stars left will take
+  unsigned long long pool_top;   // bytes of the pool given out
 };
 
 struct StarArgs {
@@ -1294,10 +1295,7 @@ static int pool_room(spnet_pc_s* pc, const StarWork& W, int64_t used, int64_t mo
     pc->pool = p;
     pc->pool_bytes = used + more;
   }
-  if (used == 0) {
-    SPNET_CUDA_TRY(cudaMemsetAsync(&W.cnt->pool_top, 0, sizeof(W.cnt->pool_top), s));
-    return SPNET_OK;
-  }
+  if (used == 0) return SPNET_OK;  // the count is zero
   const unsigned long long top = (unsigned long long)used;
   SPNET_CUDA_TRY(cudaMemcpyAsync(&W.cnt->pool_top, &top, sizeof(top), cudaMemcpyHostToDevice, s));
   SPNET_CUDA_TRY(cudaStreamSynchronize(s));  // top goes out of scope
@@ -1307,7 +1305,6 @@ static int pool_room(spnet_pc_s* pc, const StarWork& W, int64_t used, int64_t mo
 // nothing left, nothing asked for; the pool as it is
 static int clear_counts(const StarWork& W, cudaStream_t s) {
   SPNET_CUDA_TRY(cudaMemsetAsync(W.cnt, 0, offsetof(StarCount, pool_top), s));
-  SPNET_CUDA_TRY(cudaMemsetAsync(&W.cnt->pool_more, 0, sizeof(W.cnt->pool_more), s));
   return SPNET_OK;
 }
 
@@ -1418,23 +1415,21 @@ int pc_factor_stars(spnet_pc_s* pc) {
     ~Guard() { a.free_all(); }
   } guard{tmp};
   StarWork W;
-  SPNET_TRY(tmp.get(&W.noinv, pc->S));
-  SPNET_TRY(tmp.get(&W.todo, pc->S));
-  SPNET_TRY(tmp.get(&W.cnt, 1));
-  SPNET_CUDA_TRY(cudaMemsetAsync(W.noinv, 0, sizeof(int32_t) * pc->S, s));
-  fill_i32(W.todo, pc->S, STAR_TODO, s);
+  // counts and marks, all zero at first (STAR_TODO)
+  char* zero = nullptr;
+  const size_t zeros = sizeof(StarCount) + 2 * sizeof(int32_t) * (size_t)pc->S;
+  SPNET_TRY(tmp.get(&zero, zeros));
+  SPNET_CUDA_TRY(cudaMemsetAsync(zero, 0, zeros, s));
+  W.cnt = (StarCount*)zero;
+  W.noinv = (int32_t*)(zero + sizeof(StarCount));
+  W.todo = W.noinv + pc->S;
   W.left = pc->S;
   int max_row = 0;
-  {
-    int* d = nullptr;
-    SPNET_TRY(tmp.get(&d, 1));
-    SPNET_CUDA_TRY(cudaMemsetAsync(d, 0, sizeof(int), s));
-    note_launch();
-    k_max_row<<<4 * num_sms(), 256, 0, s>>>(pc->N, pc->K.ptr, d);
-    SPNET_CUDA_TRY(cudaGetLastError());
-    SPNET_CUDA_TRY(cudaMemcpyAsync(&max_row, d, sizeof(int), cudaMemcpyDeviceToHost, s));
-    SPNET_CUDA_TRY(cudaStreamSynchronize(s));
-  }
+  note_launch();
+  k_max_row<<<4 * num_sms(), 256, 0, s>>>(pc->N, pc->K.ptr, &W.cnt->max_row);
+  SPNET_CUDA_TRY(cudaGetLastError());
+  SPNET_CUDA_TRY(cudaMemcpyAsync(&max_row, &W.cnt->max_row, sizeof(int), cudaMemcpyDeviceToHost, s));
+  SPNET_CUDA_TRY(cudaStreamSynchronize(s));
   W.acap = adjacency_cap(max_row - 1, pc->d, pc->max_star);
   const int vb = pc->precision == SPNET_PREC_FP64 ? 8 : 4;
   pc->core_inv = inverted_up_to(pc->panels, pc->max_star, vb);
@@ -1464,12 +1459,11 @@ int pc_factor_stars(spnet_pc_s* pc) {
                                                                             pc->K.ptr, pc->K.col, pc->K.val, flags);
     }
     SPNET_CUDA_TRY(cudaGetLastError());
-    SPNET_CUDA_TRY(cudaMemsetAsync(W.todo, 0, sizeof(int32_t) * pc->S, s));  // STAR_DONE
+    SPNET_CUDA_TRY(cudaMemsetAsync(W.todo, STAR_DONE & 0xff, sizeof(int32_t) * pc->S, s));
     // the records of the solves: their sizes and places, the inverses of the dense blocks
     // (written into them), then the sparse entries; the set-up blobs are released
     SPNET_CUDA_TRY(cudaMemcpyAsync(lev.data(), pc->star_lev, sizeof(int32_t) * pc->S, cudaMemcpyDeviceToHost, s));
     SPNET_CUDA_TRY(cudaMemcpyAsync(nz.data(), pc->star_nnz, sizeof(int32_t) * pc->S, cudaMemcpyDeviceToHost, s));
-    SPNET_CUDA_TRY(cudaStreamSynchronize(s));
     DevArena pass;
     pass.stream = s;
     Guard pass_guard{pass};

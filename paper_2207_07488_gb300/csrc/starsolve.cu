@@ -485,6 +485,7 @@ static int records_plan_t(spnet_pc_s* pc, DevArena& tmp, const std::vector<int32
   return SPNET_OK;
 }
 
+// (lev and nz may still be on their way from the device: the wait below is theirs too)
 int star_records_plan(spnet_pc_s* pc, DevArena& tmp, const std::vector<int32_t>& lev,
                       const std::vector<int32_t>& nz, const int32_t* noinv) {
   cudaStream_t s = pc->op->stream;
@@ -992,7 +993,6 @@ int star_records_fill(spnet_pc_s* pc) {
   if (vb == 8) fill(k_record_fill<double>);
   else fill(k_record_fill<float>);
   SPNET_CUDA_TRY(cudaGetLastError());
-  SPNET_CUDA_TRY(cudaStreamSynchronize(s));
   pc->ford = pc->bord = nullptr;
   pc->core_off = nullptr;
   pc->core_kc = nullptr;
